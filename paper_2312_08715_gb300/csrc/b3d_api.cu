@@ -33,7 +33,7 @@ struct MeshRec {
     float lo[3] = {0, 0, 0}, hi[3] = {0, 0, 0};
     // voxel quads (n_quads == 0: none)
     uint2 *quads = nullptr;
-    int *class_off = nullptr;
+    int *class_off = nullptr, *tri_off = nullptr;
     float *coords = nullptr;
     int n_quads = 0, nc[3] = {0, 0, 0}, np1 = 0;
 };
@@ -316,6 +316,7 @@ MeshView view_of(const MeshRec &m) {
     v.n_quads = m.n_quads;
     v.quads = m.quads;
     v.class_off = m.class_off;
+    v.tri_off = m.tri_off;
     v.coords = m.coords;
     v.np1 = m.np1;
     return v;
@@ -904,7 +905,7 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
     //    the vertex lattice (distinct coordinates per axis), each square axis-aligned; the
     //    squares of each plane are merged into rectangles of at most 4 x 4 squares
     std::vector<uint2> h_quads;
-    std::vector<int> h_off;
+    std::vector<int> h_off, h_tri_off;
     std::vector<float> h_coords;
     int nc[3] = {0, 0, 0}, np1 = 0;
     bool quads_ok = (flags & B3D_MESH_CLOSED) && !tris.empty();
@@ -928,6 +929,7 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
             bool operator==(const QKey &o) const { return k == o.k; }
         };
         std::unordered_map<uint32_t, std::vector<std::pair<int, int>>> groups;  // key -> (tri, missing corner)
+        std::vector<uint32_t> tri_cls(tris.size(), 0);
         for (size_t i = 0; i < tris.size() && quads_ok; ++i) {
             const Tri &t = tris[i];
             const int32_t vv[3] = {t.a, t.b, t.c};
@@ -962,6 +964,7 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
             const int p = axis_idx[axis][bits(wv[3 * vv[0] + axis])];
             const uint32_t key = ((uint32_t)cls << 27) | ((uint32_t)p << 18) | ((uint32_t)b0 << 9) | (uint32_t)c0;
             groups[key].push_back({(int)i, missing});
+            tri_cls[i] = key >> 18;  // face class and plane
         }
         if (quads_ok) {
             // every unit square must be exactly two triangles split along a diagonal
@@ -1024,6 +1027,22 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
                         h_off[(size_t)cls * np1 + p] = (int)(it - rects.begin());
                     }
                 }
+                // the surface triangles by class and plane too (Morton order within a plane),
+                // with the same offsets: a renderer of triangles skips the classes turned away
+                std::vector<std::pair<uint64_t, int32_t>> order(tris.size());
+                for (size_t i = 0; i < tris.size(); ++i) order[i] = {((uint64_t)tri_cls[i] << 32) | morton(tris[i]), (int32_t)i};
+                std::sort(order.begin(), order.end());
+                for (size_t i = 0; i < tris.size(); ++i) {
+                    const Tri &t = tris[order[i].second];
+                    h_surf[i] = make_int4(t.a, t.b, t.c, t.f);
+                }
+                h_tri_off.assign((size_t)6 * np1, 0);
+                for (int cls = 0; cls < 6; ++cls)
+                    for (int p = 0; p < np1; ++p) {
+                        const uint64_t key = (uint64_t)((uint32_t)(cls << 9) | (uint32_t)std::min(p, nc[cls >> 1])) << 32;
+                        h_tri_off[(size_t)cls * np1 + p] =
+                            (int)(std::lower_bound(order.begin(), order.end(), std::make_pair(key, INT32_MIN)) - order.begin());
+                    }
                 h_quads = std::move(rects);
                 for (int a = 0; a < 3; ++a) h_coords.insert(h_coords.end(), axis_vals[a].begin(), axis_vals[a].end());
             }
@@ -1054,11 +1073,12 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
     if (rec.n_quads > 0) {
         up(&rec.quads, h_quads, "mesh rectangles");
         up(&rec.class_off, h_off, "mesh quad classes");
+        up(&rec.tri_off, h_tri_off, "mesh triangle classes");
         up(&rec.coords, h_coords, "mesh lattice");
     }
     if (st != B3D_OK) {
         dfree(ctx, rec.verts); dfree(ctx, rec.tris_surf); dfree(ctx, rec.tris_full); dfree(ctx, rec.faces);
-        dfree(ctx, rec.quads); dfree(ctx, rec.class_off); dfree(ctx, rec.coords);
+        dfree(ctx, rec.quads); dfree(ctx, rec.class_off); dfree(ctx, rec.tri_off); dfree(ctx, rec.coords);
         return st;
     }
     ctx->meshes.push_back(rec);

@@ -103,6 +103,18 @@ __device__ __forceinline__ float edge_fn(float ax, float ay, float bx, float by,
     return sw ? -e : e;
 }
 
+// An edge a->b of a rectangle or triangle staged for its pixel tests: its canonical origin (the
+// lexicographically smaller endpoint, as edge_fn) and direction, with the
+// primitive's orientation sign folded into the direction. Relative to the canonical direction
+// (from the smaller endpoint to the larger) the swap and the sign cancel:
+// (sw ? -s : s) * (sw ? a - b : b - a) = s * (b - a) exactly, since negation is exact in
+// round-to-nearest. So fmaf(E.z, py - E.y, -(E.w * (px - E.x))) equals s * edge_fn(a, b, p)
+// bit for bit (up to the sign of a zero), and the test is e >= 0.
+__device__ __forceinline__ float4 stage_edge(float ax, float ay, float bx, float by, float s) {
+    const bool sw = (bx < ax) || (bx == ax && by < ay);
+    return make_float4(sw ? bx : ax, sw ? by : ay, s * (bx - ax), s * (by - ay));
+}
+
 __device__ __forceinline__ unsigned long long pack_key(float z, unsigned id) {
     return ((unsigned long long)__float_as_uint(z) << 32) | (unsigned long long)id;
 }

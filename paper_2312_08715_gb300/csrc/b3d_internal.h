@@ -36,7 +36,9 @@ struct Cam {
 //  - verts: welded vertices (bitwise-equal positions merged), object frame.
 //  - tris_surf: the triangles that can be the nearest surface when the whole object lies
 //    beyond the near plane: for a closed outward mesh, coincident internal face pairs are
-//    removed (and back faces are skipped per hypothesis); otherwise all triangles.
+//    removed (and back faces are skipped per hypothesis); otherwise all triangles. With a
+//    rectangle representation they are sorted by face class and lattice plane, else by the
+//    Morton code of their centroids.
 //  - tris_full: every non-degenerate triangle, used when the near plane cuts the object
 //    open (then internal and back faces can be visible).
 //  - faces: the original faces on welded vertices (triangle id -> vertices).
@@ -59,7 +61,8 @@ struct MeshView {
     const int *class_off;       // [6 * (np1)]: first rectangle of class c with plane >= p
     const float *coords;        // lattice plane coordinates, x planes then y then z
     int nc[3];                  // planes per axis
-    int np1;                    // stride of class_off (max planes + 1)
+    int np1;                    // stride of class_off and tri_off (max planes + 1)
+    const int *tri_off;         // [6 * (np1)]: first surface triangle of class c with plane >= p, or NULL
 };
 
 // Windowed likelihood constants (Eq. 1 with the window of Sec. III-B).

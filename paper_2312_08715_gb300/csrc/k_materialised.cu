@@ -10,6 +10,7 @@
 #include <algorithm>
 
 #include "k_score.cuh"
+#include "k_tris.cuh"
 
 namespace b3d {
 
@@ -62,32 +63,29 @@ __global__ void __launch_bounds__(256) k_fill_bg(Cam c, const unsigned long long
 }
 
 template <class PS>
-__global__ void __launch_bounds__(kThreads) k_render_obj(SceneView S, PS P, int64_t n_hyp, float *out_depth,
-                                                         int *out_tid) {
+__global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, int64_t n_hyp, float *out_depth,
+                                                            int *out_tid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long *zb = reinterpret_cast<unsigned long long *>(smem_raw);  // [kRegionPx]
     __shared__ float s_pose[12];
     __shared__ int s_bb[4];
     __shared__ int s_flags;
+    __shared__ TriRanges s_rg;
+    __shared__ HugeQueue s_hq;
     const Cam &c = S.cam;
     const MeshView &m = S.mesh;
-    const int tid = threadIdx.x, nt = blockDim.x;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5;
     const int64_t npx = (int64_t)c.W * c.H;
     for (int64_t h = blockIdx.x; h < n_hyp; h += gridDim.x) {
         __syncthreads();
-        if (tid == 0) {
-            pose12(P, h, s_pose);
-            bool front = false;
-            s_flags = (object_bbox(m, s_pose, c, s_bb, &front) ? 1 : 0) | (front ? 4 : 0);
+        if (wid == 0) {
+            if (lane == 0) pose12(P, h, s_pose);
+            __syncwarp();
+            tri_view_warp(m, s_pose, c, lane, s_bb, &s_flags, &s_rg);
         }
         __syncthreads();
         if (!(s_flags & 1)) continue;
-        const float *pose = s_pose;
-        const bool front = (s_flags & 4) != 0;
         const int bx0 = s_bb[0], bx1 = s_bb[1], by0 = s_bb[2], by1 = s_bb[3];
-        const int4 *tris = front ? m.tris_surf : m.tris_full;
-        const int n_t = front ? m.n_surf : m.n_full;
-        const int cull = front ? m.closed : 0;
         const int tw = min(bx1 - bx0 + 1, kRegionPx);
         const int th = max(1, kRegionPx / tw);
         for (int ty0 = by0; ty0 <= by1; ty0 += th) {
@@ -95,17 +93,18 @@ __global__ void __launch_bounds__(kThreads) k_render_obj(SceneView S, PS P, int6
                 const int tx1 = min(tx0 + tw - 1, bx1), ty1 = min(ty0 + th - 1, by1);
                 const int zw = tx1 - tx0 + 1, nz = zw * (ty1 - ty0 + 1);
                 for (int i = tid; i < nz; i += nt) zb[i] = kEmptyKey;
+                if (tid == 0) s_hq.n = 0;
                 __syncthreads();
-                for (int t = tid; t < n_t; t += nt) {
-                    const int4 tr = tris[t];
-                    float4 A, B, C;
-                    tri_screen(m, tr, pose, c, A, B, C);
-                    const unsigned gid = (unsigned)(S.tri_base + tr.w);
-                    raster_tri(A, B, C, cull, tx0, tx1, ty0, ty1, c.far_z, [&](int x, int y, float z) {
-                        atomicMin(&zb[(y - ty0) * zw + (x - tx0)], pack_key(z, gid));
-                    });
+                auto store = [&](int x, int y, float z, unsigned gid) {
+                    atomicMin(&zb[(y - ty0) * zw + (x - tx0)], pack_key(z, gid));
+                };
+                for (int base = wid * 32; base < s_rg.total; base += nt)
+                    tri_batch(m, s_rg, s_flags, s_pose, S.tri_base, c, base, tx0, tx1, ty0, ty1, &s_hq, store);
+                __syncthreads();
+                if (s_hq.n > 0) {
+                    tri_huge<kThreads>(s_hq, c, store);
+                    __syncthreads();
                 }
-                __syncthreads();
                 const int dq = nt / zw, dr = nt - dq * zw;
                 int y = tid / zw, x = tid - y * zw;
                 for (int i = tid; i < nz; i += nt) {

@@ -23,21 +23,99 @@
 #include "b3d_device.cuh"
 #include "b3d_internal.h"
 #include "k_score_shapes.h"
+#include "k_tris.cuh"
 
 namespace b3d {
 
 // Camera hypotheses: every scene object k at H_h P_k, H_h the hypothesised camera_from_world
 // pose and P_k the object's world pose (the scene poses), rendered into the full image
-// (nothing is fixed, so there is no background).
+// (nothing is fixed, so there is no background). The triangles of all objects are taken 32 at
+// a time by the CTA's warps from a shared counter (k_tris.cuh).
+constexpr int kMaxCamObjects = 16;
+struct CamObject {
+    float pose[12];
+    int bb[4];
+    int flags;
+    TriRanges rg;
+};
+
+// Order of n objects by pixels of screen box per triangle, largest first (ties by index), by
+// one warp (n <= 32): batches of large triangles are handed out first, so the last batches of
+// a hypothesis are short ones (a table's batch costs 20 times a voxel mesh's).
+__device__ __forceinline__ void cam_order_warp(const CamObject *obj, int n, int lane, int *order) {
+    float key = -1.f;
+    if (lane < n && (obj[lane].flags & 1)) {
+        const int *bb = obj[lane].bb;
+        key = (float)(bb[1] - bb[0] + 1) * (float)(bb[3] - bb[2] + 1) / (float)max(obj[lane].rg.total, 1);
+    }
+    int rank = 0;
+    for (int j = 0; j < n; ++j) {
+        const float kj = __shfl_sync(0xffffffffu, key, j);
+        rank += (kj > key || (kj == key && j < lane)) ? 1 : 0;
+    }
+    if (lane < n) order[rank] = lane;
+}
+
+// Pose H_h P_k of object k in the hypothesised camera (layout of pose12), its screen box and
+// its triangle ranges, by one warp.
+__device__ __forceinline__ void cam_object_warp(CamObject &o, const MeshView &m, const float *W, const PoseList &P, int64_t h,
+                                                const Cam &c, int lane) {
+    if (lane < 12) {
+        const int r = lane < 9 ? lane / 3 : lane - 9, col = lane < 9 ? lane - 3 * r : 3;
+        const float *H = P.p + 16 * h + 4 * r;  // row r of the camera pose
+        o.pose[lane] = lane < 9 ? fmaf(H[0], W[col], fmaf(H[1], W[4 + col], H[2] * W[8 + col]))
+                                : fmaf(H[0], W[3], fmaf(H[1], W[7], fmaf(H[2], W[11], H[3])));
+    }
+    __syncwarp();
+    tri_view_warp(m, o.pose, c, lane, o.bb, &o.flags, &o.rg);
+}
+
+// The triangles of objects [0, n) over the pixels [rx0, rx1] x [ry0, ry1] into `store`;
+// *next (shared, zero before the barrier that precedes the call) hands out batches. All
+// threads of the CTA must call it; it ends with a barrier.
+template <int NT, class Store>
+__device__ __forceinline__ void cam_raster(const CamObject *obj, const int *order, int n, const MeshView *meshes,
+                                           const int *tri_base, const Cam &c, int rx0, int rx1, int ry0, int ry1, int *next, HugeQueue &hq,
+                                           Store &&store) {
+    const int lane = threadIdx.x & 31;
+    int i = 0, before = 0;  // the warp's batch is of object order[i]; batches of the objects before it
+    for (;;) {
+        int b = 0;
+        if (lane == 0) b = atomicAdd(next, 1);
+        b = __shfl_sync(0xffffffffu, b, 0);
+        while (i < n) {
+            const CamObject &o = obj[order[i]];
+            const int nb = (o.flags & 1) ? (o.rg.total + 31) >> 5 : 0;
+            if (b < before + nb) break;
+            before += nb;
+            ++i;
+        }
+        if (i >= n) break;
+        const int k = order[i];
+        const CamObject &o = obj[k];
+        const int x0 = max(rx0, o.bb[0]), x1 = min(rx1, o.bb[1]), y0 = max(ry0, o.bb[2]), y1 = min(ry1, o.bb[3]);
+        if (x0 > x1 || y0 > y1) continue;
+        tri_batch(meshes[k], o.rg, o.flags, o.pose, tri_base ? tri_base[k] : 0, c, (b - before) << 5, x0, x1, y0, y1, &hq,
+                  store);
+    }
+    __syncthreads();
+    tri_huge<NT>(hq, c, store);
+    __syncthreads();
+}
+
+// Depth and ids (64-bit keys), or depths of images whose z-buffer does not fit in shared
+// memory: screen tiles of kRegionPx pixels. Scenes of any number of objects, kMaxCamObjects
+// at a time.
 __global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshView *meshes, const int *tri_base,
                                                             const float *world, int n_obj, PoseList P, int64_t n_hyp,
                                                             float *out_depth, int *out_tid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long *zb = reinterpret_cast<unsigned long long *>(smem_raw);  // [kRegionPx]
-    __shared__ float s_pose[12];
-    __shared__ int s_bb[4];
-    __shared__ int s_flags;
-    const int tid = threadIdx.x, nt = blockDim.x;
+    __shared__ CamObject s_obj[kMaxCamObjects];
+    __shared__ int s_order[kMaxCamObjects];
+    __shared__ HugeQueue s_hq;
+    __shared__ int s_next;
+    const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
     const int64_t npx = (int64_t)c.W * c.H;
     const int tw = min(c.W, kRegionPx);
     const int th = max(1, kRegionPx / tw);
@@ -48,43 +126,21 @@ __global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshVie
                 const int zw = tx1 - tx0 + 1, zh = ty1 - ty0 + 1;
                 __syncthreads();
                 for (int i = tid; i < zw * zh; i += nt) zb[i] = kEmptyKey;
-                for (int k = 0; k < n_obj; ++k) {
-                    __syncthreads();
-                    const MeshView &m = meshes[k];
-                    if (tid == 0) {
-                        // pose of object k in the hypothesised camera: H_h P_k (rotation rows,
-                        // then translation), in the layout of pose12
-                        float Hh[12];
-                        pose12(P, h, Hh);
-                        const float *W = world + 16 * k;
-                        for (int r = 0; r < 3; ++r) {
-                            for (int col = 0; col < 3; ++col)
-                                s_pose[3 * r + col] = fmaf(Hh[3 * r], W[col], fmaf(Hh[3 * r + 1], W[4 + col], Hh[3 * r + 2] * W[8 + col]));
-                            s_pose[9 + r] = fmaf(Hh[3 * r], W[3], fmaf(Hh[3 * r + 1], W[7], fmaf(Hh[3 * r + 2], W[11], Hh[9 + r])));
-                        }
-                        bool front = false;
-                        s_flags = (object_bbox(m, s_pose, c, s_bb, &front) ? 1 : 0) | (front ? 4 : 0);
+                for (int k0 = 0; k0 < n_obj; k0 += kMaxCamObjects) {
+                    const int n = min(n_obj - k0, kMaxCamObjects);
+                    // a scene of few objects keeps its views over the tiles of a hypothesis
+                    if (n_obj > kMaxCamObjects || (ty0 == 0 && tx0 == 0)) {
+                        for (int k = wid; k < n; k += nw) cam_object_warp(s_obj[k], meshes[k0 + k], world + 16 * (k0 + k), P, h, c, lane);
+                        __syncthreads();
+                        if (wid == 0) cam_order_warp(s_obj, n, lane, s_order);
                     }
+                    if (tid == 0) { s_next = 0; s_hq.n = 0; }
                     __syncthreads();
-                    const bool front = (s_flags & 4) != 0;
-                    const int rx0 = max(tx0, s_bb[0]), rx1 = min(tx1, s_bb[1]);
-                    const int ry0 = max(ty0, s_bb[2]), ry1 = min(ty1, s_bb[3]);
-                    if (!(s_flags & 1) || rx0 > rx1 || ry0 > ry1) continue;
-                    const int4 *tris = front ? m.tris_surf : m.tris_full;
-                    const int n_t = front ? m.n_surf : m.n_full;
-                    const int cull = front ? m.closed : 0;
-                    const int base = tri_base[k];
-                    for (int t = tid; t < n_t; t += nt) {
-                        const int4 tr = tris[t];
-                        float4 A, B, C;
-                        tri_screen(m, tr, s_pose, c, A, B, C);
-                        const unsigned gid = (unsigned)(base + tr.w);
-                        raster_tri(A, B, C, cull, rx0, rx1, ry0, ry1, c.far_z, [&](int x, int y, float z) {
-                            atomicMin(&zb[(y - ty0) * zw + (x - tx0)], pack_key(z, gid));
-                        });
-                    }
+                    cam_raster<kThreads>(s_obj, s_order, n, meshes + k0, tri_base + k0, c, tx0, tx1, ty0, ty1, &s_next, s_hq,
+                                         [&](int x, int y, float z, unsigned gid) {
+                                             atomicMin(&zb[(y - ty0) * zw + (x - tx0)], pack_key(z, gid));
+                                         });
                 }
-                __syncthreads();
                 for (int i = tid; i < zw * zh; i += nt) {
                     const int gx = tx0 + i % zw, gy = ty0 + i / zw;
                     const int64_t gi = (int64_t)gy * c.W + gx;
@@ -101,55 +157,44 @@ __global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshVie
 // every object at H_h P_k in 32-bit depth bits (the same nearest depth as the 64-bit keys),
 // one pass over each object's triangles per hypothesis (the tiled kernel above sets every
 // triangle up once per screen tile).
-constexpr int kMaxCamObjects = 16;
-
 template <int NT>
 __global__ void __launch_bounds__(NT) k_render_camera_depth(Cam c, const MeshView *meshes, const float *world,
                                                             int n_obj, PoseList P, int64_t n_hyp, float *out_depth) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned *zb = reinterpret_cast<unsigned *>(smem_raw);  // [W H] depth bits
-    __shared__ float s_pose[kMaxCamObjects][12];
-    __shared__ int s_bb[kMaxCamObjects][4];
-    __shared__ int s_flags[kMaxCamObjects];
-    const int tid = threadIdx.x;
+    __shared__ CamObject s_obj[kMaxCamObjects];
+    __shared__ int s_order[kMaxCamObjects];
+    __shared__ HugeQueue s_hq;
+    __shared__ int s_next;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     const int npx = c.W * c.H;
+    const bool vec = npx % 4 == 0 && ((uintptr_t)out_depth & 15u) == 0;
+    for (int i = tid; i < npx; i += NT) zb[i] = 0xffffffffu;  // then cleared as it is read out
     for (int64_t h = blockIdx.x; h < n_hyp; h += gridDim.x) {
+        for (int k = wid; k < n_obj; k += NT / 32) cam_object_warp(s_obj[k], meshes[k], world + 16 * k, P, h, c, lane);
         __syncthreads();
-        for (int k = tid; k < n_obj; k += NT) {
-            // pose of object k in the hypothesised camera, H_h P_k, in the layout of pose12
-            float Hh[12];
-            pose12(P, h, Hh);
-            const float *W = world + 16 * k;
-            for (int r = 0; r < 3; ++r) {
-                for (int col = 0; col < 3; ++col)
-                    s_pose[k][3 * r + col] = fmaf(Hh[3 * r], W[col], fmaf(Hh[3 * r + 1], W[4 + col], Hh[3 * r + 2] * W[8 + col]));
-                s_pose[k][9 + r] = fmaf(Hh[3 * r], W[3], fmaf(Hh[3 * r + 1], W[7], fmaf(Hh[3 * r + 2], W[11], Hh[9 + r])));
-            }
-            bool front = false;
-            s_flags[k] = (object_bbox(meshes[k], s_pose[k], c, s_bb[k], &front) ? 1 : 0) | (front ? 4 : 0);
-        }
-        for (int i = tid; i < npx; i += NT) zb[i] = 0xffffffffu;
+        if (wid == 0) cam_order_warp(s_obj, n_obj, lane, s_order);
+        if (tid == 0) { s_next = 0; s_hq.n = 0; }
         __syncthreads();
-        for (int k = 0; k < n_obj; ++k) {
-            if (!(s_flags[k] & 1)) continue;
-            const MeshView &m = meshes[k];
-            const bool front = (s_flags[k] & 4) != 0;
-            const int4 *tris = front ? m.tris_surf : m.tris_full;
-            const int n_t = front ? m.n_surf : m.n_full;
-            const int cull = front ? m.closed : 0;
-            const int rx0 = s_bb[k][0], rx1 = s_bb[k][1], ry0 = s_bb[k][2], ry1 = s_bb[k][3];
-            for (int t = tid; t < n_t; t += NT) {
-                float4 A, B, C;
-                tri_screen(m, tris[t], s_pose[k], c, A, B, C);
-                raster_tri(A, B, C, cull, rx0, rx1, ry0, ry1, c.far_z,
-                           [&](int x, int y, float z) { atomicMin(&zb[y * c.W + x], __float_as_uint(z)); });
-            }
-        }
-        __syncthreads();
+        cam_raster<NT>(s_obj, s_order, n_obj, meshes, nullptr, c, 0, c.W - 1, 0, c.H - 1, &s_next, s_hq,
+                       [&](int x, int y, float z, unsigned) { atomicMin(&zb[y * c.W + x], __float_as_uint(z)); });
+        // written out and cleared for the next hypothesis by the same thread; the next
+        // hypothesis's barriers order the clears before its fragments
         float *dst = out_depth + h * npx;
-        for (int i = tid; i < npx; i += NT) {
-            const unsigned v = zb[i];
-            dst[i] = v == 0xffffffffu ? c.far_z : __uint_as_float(v);
+        auto depth_of = [&](unsigned v) { return v == 0xffffffffu ? c.far_z : __uint_as_float(v); };
+        if (vec) {
+            uint4 *z4 = reinterpret_cast<uint4 *>(zb);
+            for (int i = tid; i < npx / 4; i += NT) {
+                const uint4 v = z4[i];
+                z4[i] = make_uint4(0xffffffffu, 0xffffffffu, 0xffffffffu, 0xffffffffu);
+                reinterpret_cast<float4 *>(dst)[i] = make_float4(depth_of(v.x), depth_of(v.y), depth_of(v.z), depth_of(v.w));
+            }
+        } else {
+            for (int i = tid; i < npx; i += NT) {
+                const unsigned v = zb[i];
+                zb[i] = 0xffffffffu;
+                dst[i] = depth_of(v);
+            }
         }
     }
 }
