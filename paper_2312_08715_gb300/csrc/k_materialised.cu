@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(256) k_fill_bg(Cam c, const unsigned long long
 
 template <class PS>
 __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, int64_t n_hyp, float *out_depth,
-                                                            int *out_tid) {
+                                                         int *out_tid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned long long *zb = reinterpret_cast<unsigned long long *>(smem_raw);  // [kRegionPx]
     __shared__ float s_pose[12];
@@ -203,6 +203,89 @@ __device__ __forceinline__ void box_note(int i, int W, int &x0, int &x1, int &y0
     x0 = min(x0, x); x1 = max(x1, x); y0 = min(y0, y); y1 = max(y1, y);
 }
 
+// The pixels of a vector of four (starting at pixel i) whose bit is set in mask: one division
+// for the vector when it lies in one row.
+__device__ __forceinline__ void box_note4(int i, unsigned mask, int W, int &x0, int &x1, int &y0, int &y1) {
+    const int y = i / W, x = i - y * W;
+    if (x + 3 < W) {
+        x0 = min(x0, x + __ffs(mask) - 1); x1 = max(x1, x + 31 - __clz(mask)); y0 = min(y0, y); y1 = max(y1, y);
+    } else {
+        for (int v = 0; v < 4; ++v)
+            if ((mask >> v) & 1u) box_note(i + v, W, x0, x1, y0, y1);
+    }
+}
+
+// score_column for the 3x3 inlier ball whose window slots without a point need no test of
+// their own (r below half a metre), for the long columns of whole images: the window's three
+// rows stay in fixed registers, each new row replacing the oldest, so nothing is shifted;
+// addresses and row rays advance by one addition; the count accumulates on 2^23, whose low
+// bits are the term's index. The nine 0/1 terms add up exactly in any order, so the count, and
+// the sum, are score_column's. It takes 18% off the scoring of 200x200 images (2,048 images,
+// 0.73 -> 0.61 ms); in the fused kernel, whose columns are a few rows long, it is 0.5% slower.
+__device__ __forceinline__ float score_column_ball3(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
+                                                    const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb) {
+    const bool c0 = x > 0, c2 = x + 1 < c.W;
+    const float rx0 = ((float)(x - 1) + 0.5f - c.cx) * c.inv_fx, rx1 = ((float)x + 0.5f - c.cx) * c.inv_fx;
+    const float rx2 = ((float)(x + 1) + 0.5f - c.cx) * c.inv_fx;
+    const f32x2_t nrx01 = pk2(-rx0, -rx1), nrx22 = pk2(-rx2, -rx2);
+    const float r2b = __int_as_float(__float_as_int(L.r2) + 1) * 0x1p100f;  // (next float above r2) 2^100
+    const float *zp = zd + (ya - 1 - zy0) * zw + (x - 1 - zx0);
+    const float2 *qp = S.qe + ((int64_t)ya * c.W + x);
+    int yj = ya - 1;
+    float yf = (float)yj + 0.5f;  // exact, as are its increments
+    auto load = [&](f32x2_t &z01, float &z2, float &nry) {
+        const bool ok = (unsigned)yj < (unsigned)c.H;
+        const float a = ok && c0 ? zp[0] : -1.f, b = ok ? zp[1] : -1.f;
+        z2 = ok && c2 ? zp[2] : -1.f;
+        z01 = pk2(a, b);
+        nry = -((yf - c.cy) * c.inv_fy);
+        zp += zw;
+        yf += 1.f;
+        ++yj;
+    };
+    f32x2_t pa, pb, pc;
+    float sa, sb, sc, na, nb, nc;
+    load(pa, sa, na);
+    load(pb, sb, nb);
+    float acc = 0.f;
+    auto score = [&](float nmid) {
+        const float2 qe = *qp;  // observed depth (0: no point) and the background's term
+        qp += c.W;
+        // the observed point, formed from its depth as the observation kernel forms it
+        const float qx = __fmul_rn(qe.x, rx1), qy = __fmul_rn(qe.x, -nmid);
+        const f32x2_t qx2 = pk2(qx, qx), qy2 = pk2(qy, qy), qz2 = pk2(qe.x, qe.x);
+        // (r2+ - d2) 2^100, saturated to [0, 1], is 1 exactly when d2 <= r2 (see score_column)
+        float nf = 8388608.f;
+        auto pair = [&](f32x2_t z2, f32x2_t nrx, f32x2_t nry) {
+            const f32x2_t ex = fma2(z2, nrx, qx2), ey = fma2(z2, nry, qy2), ez = sub2(qz2, z2);
+            float d2a, d2b;
+            upk2(fma2(ex, ex, fma2(ey, ey, mul2(ez, ez))), d2a, d2b);
+            nf += __saturatef(fmaf(-d2a, 0x1p100f, r2b));
+            nf += __saturatef(fmaf(-d2b, 0x1p100f, r2b));
+        };
+        pair(pa, nrx01, pk2(na, na));
+        pair(pb, nrx01, pk2(nb, nb));
+        pair(pc, nrx01, pk2(nc, nc));
+        pair(pk2(sa, sb), nrx22, pk2(na, nb));
+        const float ex = fmaf(sc, -rx2, qx), ey = fmaf(sc, nc, qy), ez = qe.x - sc;
+        nf += __saturatef(fmaf(-fmaf(ex, ex, fmaf(ey, ey, ez * ez)), 0x1p100f, r2b));
+        const float l = lut[__float_as_int(nf) & 15];
+        if (qe.x != 0.f) acc += l - qe.y;
+    };
+    for (int left = yb - ya + 1;;) {
+        load(pc, sc, nc);
+        score(nb);
+        if (--left == 0) break;
+        load(pa, sa, na);
+        score(nc);
+        if (--left == 0) break;
+        load(pb, sb, nb);
+        score(na);
+        if (--left == 0) break;
+    }
+    return acc;
+}
+
 template <int WT, int NT, int MINB, int V, int MM>
 __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, const float *depth, const int *tid_in,
                                                           int64_t n_hyp, float *out_ll) {
@@ -216,6 +299,7 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
     for (int i = tid; i < L.n_lut; i += NT) s_lut[i] = L.lut[i];
     const int w = WT > 0 ? WT : L.w;
+    const bool ball3 = WT == 1 && L.kind == 0 && L.r2 < 0.25f;
     const int64_t npx = (int64_t)c.W * c.H;
     const float *bgd = S.bgd + (MM ? npx : 0);
     __shared__ long long s_next;
@@ -228,7 +312,30 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
         const int *tim = MM ? tid_in + h * npx : nullptr;
         // 1. the box of pixels whose depth bits differ from the background's
         int x0 = INT32_MAX, x1 = -1, y0 = INT32_MAX, y1 = -1;
-        if (V == 4) {
+        auto differs = [&](int64_t i) {
+            float d = __ldg(img + i);
+            if (MM && __ldg(tim + i) < 0) d = -1.f;
+            return __float_as_uint(d) != __float_as_uint(__ldg(bgd + i));
+        };
+        // An image that differs from the background in its first row, last row and both outer
+        // columns (a moved camera) has the whole image as its box, and needs no pass to find it.
+        bool whole = false;
+        {
+            bool e = false;
+            for (int x = tid; x < c.W; x += NT) e |= differs(x);
+            if (__syncthreads_or(e)) {
+                unsigned s = 0;
+                for (int x = tid; x < c.W; x += NT) s |= differs(npx - c.W + x) ? 1u : 0u;
+                for (int y = tid; y < c.H; y += NT) {
+                    s |= differs((int64_t)y * c.W) ? 2u : 0u;
+                    s |= differs((int64_t)y * c.W + c.W - 1) ? 4u : 0u;
+                }
+                whole = __syncthreads_or(s & 1u) && __syncthreads_or(s & 2u) && __syncthreads_or(s & 4u);
+            }
+        }
+        if (whole) {
+            x0 = 0; x1 = c.W - 1; y0 = 0; y1 = c.H - 1;
+        } else if (V == 4) {
             const int64_t n4 = npx / 4;
             const float4 *src = reinterpret_cast<const float4 *>(img);
             const int4 *tsrc = reinterpret_cast<const int4 *>(tim);
@@ -250,17 +357,15 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                     const float e[4] = {t[j].x < 0 ? -1.f : d[j].x, t[j].y < 0 ? -1.f : d[j].y,
                                         t[j].z < 0 ? -1.f : d[j].z, t[j].w < 0 ? -1.f : d[j].w};
                     const float b[4] = {g[j].x, g[j].y, g[j].z, g[j].w};
+                    unsigned mask = 0;
 #pragma unroll
-                    for (int v = 0; v < 4; ++v)
-                        if (__float_as_uint(e[v]) != __float_as_uint(b[v])) box_note((int)(4 * k + v), c.W, x0, x1, y0, y1);
+                    for (int v = 0; v < 4; ++v) mask |= __float_as_uint(e[v]) != __float_as_uint(b[v]) ? 1u << v : 0u;
+                    if (mask) box_note4((int)(4 * k), mask, c.W, x0, x1, y0, y1);
                 }
             }
         } else {
-            for (int64_t k = tid; k < npx; k += NT) {
-                float d = __ldg(img + k);
-                if (MM && __ldg(tim + k) < 0) d = -1.f;
-                if (__float_as_uint(d) != __float_as_uint(__ldg(bgd + k))) box_note((int)k, c.W, x0, x1, y0, y1);
-            }
+            for (int64_t k = tid; k < npx; k += NT)
+                if (differs(k)) box_note((int)k, c.W, x0, x1, y0, y1);
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
@@ -293,7 +398,7 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                         const int dq = NT / zw, dr = NT - dq * zw;
                         int y = tid / zw, x = tid - y * zw;
                         for (int i = tid; i < nz; i += NT) {
-                            const int64_t gi = (int64_t)(zy0 + y) * c.W + (zx0 + x);
+                            const int gi = (zy0 + y) * c.W + (zx0 + x);  // an image has at most 2^26 pixels
                             float d = img[gi];
                             if (MM && tim[gi] < 0) d = -1.f;
                             zd[i] = d;
@@ -312,8 +417,10 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                         if (seg < nseg && col < tww) {
                             const int ya = ty0 + seg * rps, yb = min(ya + rps - 1, ty1);
                             if (ya <= yb)
-                                acc += score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, nullptr,
-                                                        nullptr);
+                                acc += WT == 1 && ball3
+                                           ? score_column_ball3(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb)
+                                           : score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, nullptr,
+                                                              nullptr);
                         }
                     } else {
                         const int n_t = tww * thh;
@@ -360,12 +467,15 @@ static int persistent_grid(K kernel, int threads, int smem, int64_t n, int grid)
 }
 
 // Launch shape of the fused materialised kernels: 128-thread CTAs; register caps from
-// launch-bound sweeps on the 160x120 tabletop stage (145,800 images): the renderer at 8
-// CTAs per SM (64 registers; 3.64 against 3.77 ms at 6), the ball scorer at 10 (48
-// registers, no spills; 2.32 against 2.59 ms at 6, 2.44 at 8, 2.53 at 12, where it spills).
+// launch-bound sweeps: the renderer at 8 CTAs per SM on the 160x120 tabletop stage (145,800
+// images; 64 registers; 3.64 against 3.77 ms at 6). The 3x3 scorer of images that differ from
+// the reference around one object streams most of its pixels and wants 8 CTAs (render and
+// score of 20,000 images 795 us; 10: 799, 7: 809); images of the whole scene moved (no object
+// slot: a camera's) are scored everywhere and want registers: 7 (camera call of 2,048 images
+// of 200x200 1,638 us; 8: 1,735, 10: 1,755, 6: 1,637).
 constexpr int kMatNT = 128, kRenderMinB = 8;
 template <int WT>
-constexpr int score_fused_minb() { return WT == 1 ? 10 : 6; }
+constexpr int score_fused_minb(bool whole) { return WT == 1 ? (whole ? 7 : 8) : 6; }
 
 int launch_render_list(const SceneView &sv, PoseList P, int64_t n, float *depth, int *tid, int grid, cudaStream_t s) {
     if (n <= 0) return 0;
@@ -391,13 +501,13 @@ int launch_render_list(const SceneView &sv, PoseList P, int64_t n, float *depth,
     return 1;
 }
 
-template <int WT>
+template <int WT, bool WHOLE>
 static void launch_score_fused(const SceneView &sv, const Lik &L, const float *depth, const int *tid, int64_t n,
                                float *ll, int grid, cudaStream_t s) {
     const int64_t npx = (int64_t)sv.cam.W * sv.cam.H;
     const bool mm = L.miss_mode == 1;
     const bool vec = npx % 4 == 0 && aligned16p(depth) && (!mm || aligned16p(tid));
-    constexpr int MB = score_fused_minb<WT>();
+    constexpr int MB = score_fused_minb<WT>(WHOLE);
     auto kern = vec ? (mm ? k_score_fused<WT, kMatNT, MB, 4, 1> : k_score_fused<WT, kMatNT, MB, 4, 0>)
                     : (mm ? k_score_fused<WT, kMatNT, MB, 1, 1> : k_score_fused<WT, kMatNT, MB, 1, 0>);
     if (sv.work) cudaMemsetAsync(sv.work, 0, sizeof(unsigned long long), s);
@@ -407,9 +517,11 @@ static void launch_score_fused(const SceneView &sv, const Lik &L, const float *d
 int launch_score_depth(const SceneView &sv, const Lik &L, const float *depth, const int *tid, int64_t n, float *ll,
                        int grid, cudaStream_t s) {
     if (n <= 0) return 0;
-    if (L.w == 1) launch_score_fused<1>(sv, L, depth, tid, n, ll, grid, s);
-    else if (L.w == 2) launch_score_fused<2>(sv, L, depth, tid, n, ll, grid, s);
-    else launch_score_fused<0>(sv, L, depth, tid, n, ll, grid, s);
+    const bool whole = sv.mesh.n_full <= 0;  // no object slot
+    if (L.w == 1 && whole) launch_score_fused<1, true>(sv, L, depth, tid, n, ll, grid, s);
+    else if (L.w == 1) launch_score_fused<1, false>(sv, L, depth, tid, n, ll, grid, s);
+    else if (L.w == 2) launch_score_fused<2, false>(sv, L, depth, tid, n, ll, grid, s);
+    else launch_score_fused<0, false>(sv, L, depth, tid, n, ll, grid, s);
     return 1;
 }
 
