@@ -122,7 +122,8 @@ __global__ void k_set16(float *dst, F16 src) {
 // ------------------------------------------------------------------------------------------
 // fused log-sum-exp + categorical resampling
 // ------------------------------------------------------------------------------------------
-constexpr int kLseThreads = 256;
+constexpr int kLseThreads = 256;  // threads that share a block's chunk and the chunk prefix (their sums' order)
+constexpr int kLseBlock = 512;    // threads of a block: the last block's draws want warps
 constexpr int kLseMaxBlocks = 1024;
 constexpr int kLseMinChunk = 512;
 
@@ -132,18 +133,21 @@ __device__ __forceinline__ float lse_weight(float x, float m) {
 
 // Phase A (every block): chunk max m_b and s_b = sum exp(ll - m_b) -> part[b].
 // Phase B (the last block to finish, by an atomic ticket; no block waits on another):
-// global max M, S = sum_b s_b exp(m_b - M), chunk prefix sums, logZ = M + log S, then each
-// draw k: t = u_k S, chunk by binary search on the chunk prefix, element by a warp scan of
-// exp(ll - M) within the chunk (first inclusive prefix > t). The counter is reset for the
-// next launch.
+// global max M, S = sum_b s_b exp(m_b - M), chunk prefix sums, logZ = M + log S; then the
+// draws, kLseBlock at a time: a thread forms each draw's t = u_k S and finds its chunk by
+// binary search on the chunk prefix, and a warp finds the element (first inclusive prefix > t
+// in the chunk). The counter is reset for the next launch.
+// It is latency that bounds the call (584 KB of scores; a chain of reductions, then the
+// draws), so the draws' parts are spread over the block: with 8 warps that each formed,
+// searched and scanned 13 of 100 draws one after another, 145,800 scores took 57 us;
+// now 20 us (the kernel, ncu), and 6,250 scores with 16 draws 9 us (12 before).
 struct LseShared {
     float red[kLseThreads / 32];
     float w[kLseMaxBlocks];
     float pre[kLseMaxBlocks];  // exclusive prefix of w
-    float cp[kLseThreads / 32][kLseMinChunk];         // per warp: inclusive prefix of one chunk,
-    float cl[kLseThreads / 32][kLseMinChunk];         // its scores
-    unsigned cm[kLseThreads / 32][kLseMinChunk / 32];  // and which of its weights are positive
-    float M, S;
+    float t[kLseBlock];        // of the draws of a pass: the target,
+    int b[kLseBlock];          // and its chunk, then its element (-1: none, -2: another rank's draw)
+    float S;
     bool last;
 };
 
@@ -158,59 +162,80 @@ __device__ __forceinline__ void lse_body(LseShared &sh, int bid, int nb, const f
                                          float *logz, int *idx, float *logq, int *err,
                                          const LseShard *shard = nullptr) {
     float *s_red = sh.red, *s_w = sh.w, *s_pre = sh.pre;
-    float &s_M = sh.M, &s_S = sh.S;
-    bool &s_last = sh.last;
-    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = kLseThreads / 32;
+    const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    constexpr int nw = kLseThreads / 32;
+    const bool works = tid < kLseThreads;  // whole warps
     const int64_t b0 = (int64_t)bid * chunk, b1 = std::min<int64_t>(n, b0 + chunk);
 
-    // phase A
-    float mx = -INFINITY;
-    for (int64_t i = b0 + tid; i < b1; i += kLseThreads) mx = fmaxf(mx, ll[i]);
-    for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-    if (lane == 0) s_red[wid] = mx;
-    __syncthreads();
-    if (tid == 0) {
-        float v = -INFINITY;
-        for (int k = 0; k < nw; ++k) v = fmaxf(v, s_red[k]);
-        s_M = v;
+    // phase A; a chunk of up to two scores a thread stays in registers
+    const bool held = chunk <= 2 * kLseThreads;
+    float x0 = -INFINITY, x1 = -INFINITY, mx = -INFINITY;
+    if (works) {
+        if (held) {
+            if (b0 + tid < b1) x0 = ll[b0 + tid];
+            if (b0 + tid + kLseThreads < b1) x1 = ll[b0 + tid + kLseThreads];
+            mx = fmaxf(fmaxf(mx, x0), x1);
+        } else {
+            for (int64_t i = b0 + tid; i < b1; i += kLseThreads) mx = fmaxf(mx, ll[i]);
+        }
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+        if (lane == 0) s_red[wid] = mx;
     }
     __syncthreads();
-    const float mb = s_M;
-    float sm = 0.f;
-    for (int64_t i = b0 + tid; i < b1; i += kLseThreads) sm += lse_weight(ll[i], mb);
-    for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, o);
+    float mb = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < nw; ++k) mb = fmaxf(mb, s_red[k]);
     __syncthreads();
-    if (lane == 0) s_red[wid] = sm;
+    if (works) {
+        float sm = 0.f;
+        if (held) {
+            if (b0 + tid < b1) sm += lse_weight(x0, mb);
+            if (b0 + tid + kLseThreads < b1) sm += lse_weight(x1, mb);
+        } else {
+            for (int64_t i = b0 + tid; i < b1; i += kLseThreads) sm += lse_weight(ll[i], mb);
+        }
+        for (int o = 16; o > 0; o >>= 1) sm += __shfl_xor_sync(0xffffffffu, sm, o);
+        if (lane == 0) s_red[wid] = sm;
+    }
     __syncthreads();
     if (tid == 0) {
         float v = 0.f;
+#pragma unroll
         for (int k = 0; k < nw; ++k) v += s_red[k];
         part[bid] = make_float2(mb, v);
         __threadfence();
         const unsigned ticket = atomicAdd(counter, 1u);
-        s_last = ticket == (unsigned)nb - 1;
+        sh.last = ticket == (unsigned)nb - 1;
     }
     __syncthreads();
-    if (!s_last) return;
+    if (!sh.last) return;
     __threadfence();
 
     // phase B
     const int B = nb;
+    constexpr int kRuns = kLseMaxBlocks / kLseThreads;
+    float2 pt[kRuns];  // the partials of chunks tid, tid + 256, ...
     float gm = -INFINITY;
-    for (int b = tid; b < B; b += kLseThreads) gm = fmaxf(gm, __ldcg(&part[b].x));
-    for (int o = 16; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
-    if (lane == 0) s_red[wid] = gm;
-    __syncthreads();
-    if (tid == 0) {
-        float v = -INFINITY;
-        for (int k = 0; k < nw; ++k) v = fmaxf(v, s_red[k]);
-        s_M = v;
+    if (works) {
+#pragma unroll
+        for (int r = 0; r < kRuns; ++r) {
+            const int b = tid + r * kLseThreads;
+            pt[r] = b < B ? __ldcg(&part[b]) : make_float2(-INFINITY, 0.f);
+            gm = fmaxf(gm, pt[r].x);
+        }
+        for (int o = 16; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+        if (lane == 0) s_red[wid] = gm;
     }
     __syncthreads();
-    const float M = s_M;
-    for (int b = tid; b < B; b += kLseThreads) {
-        const float2 p = __ldcg(&part[b]);
-        s_w[b] = (p.x > -INFINITY && M > -INFINITY) ? p.y * __expf(p.x - M) : 0.f;
+    float M = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < nw; ++k) M = fmaxf(M, s_red[k]);
+    if (works) {
+#pragma unroll
+        for (int r = 0; r < kRuns; ++r) {
+            const int b = tid + r * kLseThreads;
+            if (b < B) s_w[b] = (pt[r].x > -INFINITY && M > -INFINITY) ? pt[r].y * __expf(pt[r].x - M) : 0.f;
+        }
     }
     __syncthreads();
     {
@@ -219,162 +244,179 @@ __device__ __forceinline__ void lse_body(LseShared &sh, int bid, int nb, const f
         // order), and each thread writes its run's prefixes
         const int R = (B + kLseThreads - 1) / kLseThreads;
         const int r0 = min(tid * R, B), r1 = min(r0 + R, B);
-        float run = 0.f;
-        for (int b = r0; b < r1; ++b) run += s_w[b];
-        float inc = run;
-        for (int o = 1; o < 32; o <<= 1) {
-            const float up = __shfl_up_sync(0xffffffffu, inc, o);
-            if (lane >= o) inc += up;
-        }
-        if (lane == 31) s_red[wid] = inc;
-        __syncthreads();
-        if (tid == 0) {
-            float acc = 0.f;
-            for (int k = 0; k < nw; ++k) {
-                const float v = s_red[k];
-                s_red[k] = acc;
-                acc += v;
+        float run = 0.f, inc = 0.f;
+        if (works) {
+            for (int b = r0; b < r1; ++b) run += s_w[b];
+            inc = run;
+            for (int o = 1; o < 32; o <<= 1) {
+                const float up = __shfl_up_sync(0xffffffffu, inc, o);
+                if (lane >= o) inc += up;
             }
-            s_S = acc;
-            *counter = 0u;
-            *logz = (M > -INFINITY) ? M + __logf(acc) : -INFINITY;
-            if (!(M > -INFINITY) && m > 0 && !shard) atomicOr(err, 4);
+            if (lane == 31) s_red[wid] = inc;
         }
         __syncthreads();
-        float acc = s_red[wid] + (inc - run);
-        for (int b = r0; b < r1; ++b) {
-            s_pre[b] = acc;
-            acc += s_w[b];
+        if (works) {
+            float before = 0.f, acc = 0.f;  // of the warps before this one, and of all, in order
+#pragma unroll
+            for (int k = 0; k < nw; ++k) {
+                if (k == wid) before = acc;
+                acc += s_red[k];
+            }
+            if (tid == 0) {
+                sh.S = acc;
+                *counter = 0u;
+                *logz = (M > -INFINITY) ? M + __logf(acc) : -INFINITY;
+                if (!(M > -INFINITY) && m > 0 && !shard) atomicOr(err, 4);
+            }
+            acc = before + (inc - run);
+            for (int b = r0; b < r1; ++b) {
+                s_pre[b] = acc;
+                acc += s_w[b];
+            }
         }
     }
     __syncthreads();
-    const float S = s_S;
+    const float S = sh.S;
     const float Z = shard ? shard->logz : ((M > -INFINITY) ? M + __logf(S) : -INFINITY);
     const long long ibase = shard ? shard->base : 0;
-    int cached = -1;  // the chunk whose prefix this warp holds
-    for (int k = wid; k < m; k += nw) {
-        if (!(M > -INFINITY)) {
-            if (lane == 0) { idx[k] = -1; logq[k] = -INFINITY; }
-            continue;
+    if (!(M > -INFINITY)) {
+        for (int k = tid; k < m; k += kLseBlock) {
+            idx[k] = -1;
+            logq[k] = -INFINITY;
         }
-        const U64x4 r = philox4x64((unsigned long long)k, (unsigned long long)(unsigned)stage, 0ull, 0ull, seed, 0ull);
-        float t;
-        if (shard) {
-            const double u = (double)(r.v[0] >> 40) * (1.0 / 16777216.0);  // the same 24-bit uniform, exact
-            if (!(u >= shard->before && u < shard->before + shard->mass)) {
-                if (lane == 0) { idx[k] = -1; logq[k] = -INFINITY; }
+        return;
+    }
+    constexpr int G = kLseMinChunk / 32;
+    int cached = -1;  // the chunk this warp holds:
+    float cp[G];         // the inclusive prefix of its weights, element 32 j + lane,
+    unsigned pos[G];     // and which of them are positive
+#pragma unroll
+    for (int j = 0; j < G; ++j) { cp[j] = 0.f; pos[j] = 0u; }
+    for (int k0 = 0; k0 < m; k0 += kLseBlock) {
+        if (k0 + tid < m) {
+            const U64x4 r = philox4x64((unsigned long long)(k0 + tid), (unsigned long long)(unsigned)stage, 0ull, 0ull, seed,
+                                       0ull);
+            float t = 0.f;
+            int b = 0;
+            if (shard) {
+                const double u = (double)(r.v[0] >> 40) * (1.0 / 16777216.0);  // the same 24-bit uniform, exact
+                if (!(u >= shard->before && u < shard->before + shard->mass)) {
+                    b = -2;
+                } else {
+                    t = (float)((u - shard->before) / shard->mass) * S;
+                }
+            } else {
+                t = uniform24(r.v[0]) * S;
+            }
+            if (b == 0) {
+                // first chunk whose inclusive prefix exceeds t; if rounding leaves none, the
+                // last chunk with weight
+                int lo = 0, hi = B - 1;
+                while (lo < hi) {
+                    const int mid = (lo + hi) >> 1;
+                    if (s_pre[mid] + s_w[mid] > t) hi = mid; else lo = mid + 1;
+                }
+                b = lo;
+                if (!(s_pre[b] + s_w[b] > t)) {
+                    b = B - 1;
+                    while (b > 0 && s_w[b] == 0.f) --b;
+                }
+            }
+            sh.t[tid] = t;
+            sh.b[tid] = b;
+        }
+        __syncthreads();
+        const int k1 = min(k0 + kLseBlock, m);
+        for (int k = k0 + wid; k < k1; k += kLseBlock / 32) {
+            const float t = sh.t[k - k0];
+            const int b = sh.b[k - k0];
+            if (b < 0) continue;
+            const int64_t e0 = (int64_t)b * chunk, e1 = std::min<int64_t>(n, e0 + chunk);
+            if (chunk <= kLseMinChunk) {
+                // the chunk's inclusive prefix (groups of 32, a warp scan each, added in order:
+                // the sums of the streaming search below), kept for the warp's next draws
+                const int len = (int)(e1 - e0);
+                if (b != cached) {
+                    float inc[G];
+#pragma unroll
+                    for (int j = 0; j < G; ++j) {  // every load of the chunk in flight together
+                        const int i = 32 * j + lane;
+                        inc[j] = i < len ? __ldcg(&ll[e0 + i]) : -INFINITY;
+                    }
+#pragma unroll
+                    for (int j = 0; j < G; ++j) {
+                        inc[j] = lse_weight(inc[j], M);
+                        pos[j] = __ballot_sync(0xffffffffu, inc[j] > 0.f);
+                    }
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {  // the groups' scans step together
+#pragma unroll
+                        for (int j = 0; j < G; ++j) {
+                            const float up = __shfl_up_sync(0xffffffffu, inc[j], o);
+                            if (lane >= o) inc[j] += up;
+                        }
+                    }
+                    float c1 = s_pre[b];
+#pragma unroll
+                    for (int j = 0; j < G; ++j) {
+                        cp[j] = c1 + inc[j];
+                        c1 += __shfl_sync(0xffffffffu, inc[j], 31);
+                    }
+                    cached = b;
+                }
+                // first element with a positive weight whose inclusive prefix exceeds t (the
+                // prefix never decreases); if rounding leaves none, the last positive one
+                int found = -1, last_pos = -1;
+#pragma unroll
+                for (int j = 0; j < G; ++j) {
+                    const unsigned hit = __ballot_sync(0xffffffffu, cp[j] > t) & pos[j];
+                    if (hit && found < 0) found = 32 * j + __ffs(hit) - 1;
+                    if (pos[j]) last_pos = 32 * j + 31 - __clz(pos[j]);
+                }
+                if (found < 0) found = last_pos;
+                if (lane == 0) sh.b[k - k0] = found >= 0 ? (int)(e0 + found) : -1;
                 continue;
             }
-            t = (float)((u - shard->before) / shard->mass) * S;
-        } else {
-            t = uniform24(r.v[0]) * S;
-        }
-        // first chunk whose inclusive prefix exceeds t; if rounding leaves none, the last
-        // chunk with weight
-        int lo = 0, hi = B - 1;
-        while (lo < hi) {
-            const int mid = (lo + hi) >> 1;
-            if (s_pre[mid] + s_w[mid] > t) hi = mid; else lo = mid + 1;
-        }
-        int b = lo;
-        if (!(s_pre[b] + s_w[b] > t)) {
-            b = B - 1;
-            while (b > 0 && s_w[b] == 0.f) --b;
-        }
-        const int64_t e0 = (int64_t)b * chunk, e1 = std::min<int64_t>(n, e0 + chunk);
-        if (chunk <= kLseMinChunk) {
-            // the chunk's inclusive prefix (the same groups of 32 and the same warp scans as
-            // the streaming search below, so the same sums) and its positive weights, kept
-            // per warp: further draws in the chunk only search shared memory
-            float *cp = sh.cp[wid], *cl = sh.cl[wid];
-            unsigned *cm = sh.cm[wid];
-            const int len = (int)(e1 - e0);
-            if (b != cached) {
-                constexpr int G = kLseMinChunk / 32;
-                float lv[G];  // every load of the chunk in flight before the scan
+            float c0 = s_pre[b];
+            int64_t found = -1, last_pos = -1;
+            // 128 elements per pass, four independent loads in flight per lane
+            for (int64_t base = e0; base < e1 && found < 0; base += 128) {
+                float wv[4];
 #pragma unroll
-                for (int j = 0; j < G; ++j) {
-                    const int i = 32 * j + lane;
-                    lv[j] = i < len ? __ldcg(&ll[e0 + i]) : -INFINITY;
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t i = base + 32 * u + lane;
+                    wv[u] = i < e1 ? lse_weight(__ldcg(&ll[i]), M) : 0.f;
                 }
-                float c1 = s_pre[b];
 #pragma unroll
-                for (int j = 0; j < G; ++j) {
-                    const int i = 32 * j + lane;
-                    if (32 * j >= len) break;
-                    const float wv = i < len ? lse_weight(lv[j], M) : 0.f;
-                    float inc = wv;
+                for (int u = 0; u < 4; ++u) {
+                    const int64_t i = base + 32 * u + lane;
+                    float inc = wv[u];
                     for (int o = 1; o < 32; o <<= 1) {
                         const float up = __shfl_up_sync(0xffffffffu, inc, o);
                         if (lane >= o) inc += up;
                     }
-                    if (i < len) {
-                        cp[i] = c1 + inc;
-                        cl[i] = lv[j];
+                    const unsigned hit = __ballot_sync(0xffffffffu, i < e1 && wv[u] > 0.f && c0 + inc > t);
+                    const unsigned ps = __ballot_sync(0xffffffffu, i < e1 && wv[u] > 0.f);
+                    if (found < 0) {
+                        if (ps) last_pos = base + 32 * u + 31 - __clz(ps);
+                        if (hit) found = base + 32 * u + __ffs(hit) - 1;
                     }
-                    const unsigned pos = __ballot_sync(0xffffffffu, i < len && wv > 0.f);
-                    if (lane == 0) cm[j] = pos;
-                    c1 += __shfl_sync(0xffffffffu, inc, 31);
+                    c0 += __shfl_sync(0xffffffffu, inc, 31);
                 }
-                cached = b;
-                __syncwarp();
             }
-            if (lane == 0) {
-                // first element with a positive weight whose inclusive prefix exceeds t (the
-                // prefix never decreases); if rounding leaves none, the last positive one
-                int lo = 0, hi = len;
-                while (lo < hi) {
-                    const int mid = (lo + hi) >> 1;
-                    if (cp[mid] > t) hi = mid; else lo = mid + 1;
-                }
-                int found = -1;
-                for (int i = lo; i < len; ++i)
-                    if ((cm[i >> 5] >> (i & 31)) & 1u) { found = i; break; }
-                if (found < 0)
-                    for (int i = len - 1; i >= 0; --i)
-                        if ((cm[i >> 5] >> (i & 31)) & 1u) { found = i; break; }
-                idx[k] = found >= 0 ? (int)(ibase + e0 + found) : -1;
-                logq[k] = found >= 0 ? cl[found] - Z : -INFINITY;
-            }
-            __syncwarp();
-            continue;
+            if (found < 0) found = last_pos;
+            if (lane == 0) sh.b[k - k0] = (int)found;
         }
-        float c0 = s_pre[b];
-        int64_t found = -1, last_pos = -1;
-        // 128 elements per pass, four independent loads in flight per lane
-        for (int64_t base = e0; base < e1 && found < 0; base += 128) {
-            float wv[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = base + 32 * u + lane;
-                wv[u] = i < e1 ? lse_weight(__ldcg(&ll[i]), M) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                const int64_t i = base + 32 * u + lane;
-                float inc = wv[u];
-                for (int o = 1; o < 32; o <<= 1) {
-                    const float up = __shfl_up_sync(0xffffffffu, inc, o);
-                    if (lane >= o) inc += up;
-                }
-                const unsigned hit = __ballot_sync(0xffffffffu, i < e1 && wv[u] > 0.f && c0 + inc > t);
-                const unsigned pos = __ballot_sync(0xffffffffu, i < e1 && wv[u] > 0.f);
-                if (found < 0) {
-                    if (pos) last_pos = base + 32 * u + 31 - __clz(pos);
-                    if (hit) found = base + 32 * u + __ffs(hit) - 1;
-                }
-                c0 += __shfl_sync(0xffffffffu, inc, 31);
-            }
-        }
-        if (found < 0) found = last_pos;
-        if (lane == 0) {
-            idx[k] = found >= 0 ? (int)(ibase + found) : -1;
-            logq[k] = found >= 0 ? __ldcg(&ll[found]) - Z : -INFINITY;
+        __syncthreads();
+        if (k0 + tid < m) {
+            const int f = sh.b[tid];
+            idx[k0 + tid] = f >= 0 ? (int)(ibase + f) : -1;
+            logq[k0 + tid] = f >= 0 ? __ldcg(&ll[f]) - Z : -INFINITY;
         }
     }
 }
 
-__global__ void __launch_bounds__(kLseThreads) k_lse_resample(const float *ll, int64_t n, int chunk, int m,
+__global__ void __launch_bounds__(kLseBlock, 2) k_lse_resample(const float *ll, int64_t n, int chunk, int m,
                                                               unsigned long long seed, int stage, float2 *part,
                                                               unsigned *counter, float *logz, int *idx, float *logq,
                                                               int *err) {
@@ -383,7 +425,7 @@ __global__ void __launch_bounds__(kLseThreads) k_lse_resample(const float *ll, i
 }
 
 // One rank's shard of a categorical split over ranks (see lse_body).
-__global__ void __launch_bounds__(kLseThreads) k_lse_shard(const float *ll, int64_t n, int chunk, int m,
+__global__ void __launch_bounds__(kLseBlock, 2) k_lse_shard(const float *ll, int64_t n, int chunk, int m,
                                                            unsigned long long seed, int stage, LseShard shard,
                                                            float2 *part, unsigned *counter, float *logz, int *idx,
                                                            float *logq, int *err) {
@@ -393,7 +435,7 @@ __global__ void __launch_bounds__(kLseThreads) k_lse_shard(const float *ll, int6
 
 // Batched: the blocks of every scene's score vector in one grid; block_begin[i] is the
 // first block of item i.
-__global__ void __launch_bounds__(kLseThreads) k_lse_multi(const LseItem *items, int n_items, const int *block_begin,
+__global__ void __launch_bounds__(kLseBlock, 2) k_lse_multi(const LseItem *items, int n_items, const int *block_begin,
                                                            int *err) {
     __shared__ LseShared sh;
     __shared__ int s_it;
@@ -417,7 +459,7 @@ void launch_lse_resample(const float *ll, int64_t n, int m, uint64_t seed, int s
                          float *logz, int *idx, float *logq, int *err, cudaStream_t s) {
     const int B = lse_blocks(n);
     const int chunk = (int)((n + B - 1) / B);
-    k_lse_resample<<<B, kLseThreads, 0, s>>>(ll, n, chunk, m, (unsigned long long)seed, stage, part, counter, logz, idx,
+    k_lse_resample<<<B, kLseBlock, 0, s>>>(ll, n, chunk, m, (unsigned long long)seed, stage, part, counter, logz, idx,
                                              logq, err);
 }
 
@@ -425,7 +467,7 @@ void launch_lse_shard(const float *ll, int64_t n, int m, uint64_t seed, int stag
                       unsigned *counter, float *logz, int *idx, float *logq, int *err, cudaStream_t s) {
     const int B = lse_blocks(n);
     const int chunk = (int)((n + B - 1) / B);
-    k_lse_shard<<<B, kLseThreads, 0, s>>>(ll, n, chunk, m, (unsigned long long)seed, stage, shard, part, counter, logz,
+    k_lse_shard<<<B, kLseBlock, 0, s>>>(ll, n, chunk, m, (unsigned long long)seed, stage, shard, part, counter, logz,
                                           idx, logq, err);
 }
 
@@ -539,7 +581,7 @@ void launch_c2f_select(const float *ll, const int *idx, int m, PoseGrid P, const
 void launch_lse_multi(const LseItem *items, int n_items, int total_blocks, const int *block_begin, int *err,
                       cudaStream_t s) {
     if (n_items <= 0 || total_blocks <= 0) return;
-    k_lse_multi<<<total_blocks, kLseThreads, 0, s>>>(items, n_items, block_begin, err);
+    k_lse_multi<<<total_blocks, kLseBlock, 0, s>>>(items, n_items, block_begin, err);
 }
 
 void launch_select_multi(const SelectItem *items, int n_items, int last, int stage, cudaStream_t s) {
