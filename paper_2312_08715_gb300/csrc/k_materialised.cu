@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
         if (x1 >= 0) {
             const int sx0 = max(x0 - w, 0), sx1 = min(x1 + w, c.W - 1);
             const int sy0 = max(y0 - w, 0), sy1 = min(y1 + w, c.H - 1);
-            const int tw = min(min(sx1 - sx0 + 1, S.tile_w), REG / (1 + 2 * w) - 2 * w);
+            const int tw = min(min(sx1 - sx0 + 1, min(S.tile_w, NT)), REG / (1 + 2 * w) - 2 * w);
             const int th = max(1, REG / (tw + 2 * w) - 2 * w);
             for (int ty0 = sy0; ty0 <= sy1; ty0 += th) {
                 for (int tx0 = sx0; tx0 <= sx1; tx0 += tw) {

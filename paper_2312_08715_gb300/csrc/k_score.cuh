@@ -376,8 +376,9 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
     const int sx0 = max(bx0 - w, 0), sx1 = min(bx1 + w, c.W - 1);
     const int sy0 = max(by0 - w, 0), sy1 = min(by1 + w, c.H - 1);
     const int sw = sx1 - sx0 + 1;
-    // the tile plus its halo must fit the region even one row high: (tw + 2w)(1 + 2w) <= REG
-    const int tw = min(min(sw, S.tile_w), REG / (1 + 2 * w) - 2 * w);
+    // the tile plus its halo must fit the region even one row high: (tw + 2w)(1 + 2w) <= REG;
+    // the column scorers give each column of a tile a thread
+    const int tw = min(min(sw, TAGS ? S.tile_w : min(S.tile_w, NT)), REG / (1 + 2 * w) - 2 * w);
     const int th = max(1, REG / (tw + 2 * w) - 2 * w);
     for (int ty0 = sy0; ty0 <= sy1; ty0 += th) {
         for (int tx0 = sx0; tx0 <= sx1; tx0 += tw) {
