@@ -270,7 +270,9 @@ b3d_status b3d_enumerate_c2f(b3d_ctx *ctx, int32_t obj_slot, const float *centre
  * persistent launch whose CTAs take batch_chunk hypotheses at a time from a work queue over
  * (scene, hypothesis chunk). Items may differ in image size, meshes, object slot and
  * hypothesis count; the likelihood is shared (its frustum volume is each scene's own).
- * Scores equal those of b3d_score_batch on each scene alone. The owner's context supplies
+ * Scores equal those of b3d_score_batch on each scene alone (bit for bit under the same
+ * b3d_set_tuning; a context that was not tuned picks its launch shape by the size of the work,
+ * and shapes differ in FP32 summation order). The owner's context supplies
  * the launch shape (b3d_tuning) and the scratch; scratch is sized on first use, after
  * which the call can be captured into a CUDA graph (it allocates nothing and only copies its
  * descriptors from pinned host memory). */
@@ -381,7 +383,10 @@ b3d_status b3d_score_noise_batch(b3d_ctx *ctx, int32_t obj_slot, int64_t n_hyp, 
  * of this implementation). tile_w: widest screen tile in pixels (8..256); cta_threads: 32,
  * 64, 128 or 256 (one hypothesis per CTA at a time); ctas_per_sm: CTAs resident per SM
  * (0 = as many as fit); high_occupancy: 1 selects the build whose registers are capped so
- * that more CTAs fit on an SM, 0 the regular one; batch_chunk (1..1024): see b3d_score_multi. */
+ * that more CTAs fit on an SM, 0 the regular one; batch_chunk (1..1024): see b3d_score_multi.
+ * Until b3d_set_tuning or an autotuner is called on a context, its score launches with half
+ * windows 1 and 2 of voxel meshes take a CTA size and tile width chosen by the size of the
+ * object, the image and the batch; b3d_get_tuning then reports the general default. */
 typedef struct {
     int32_t tile_w;
     int32_t cta_threads;

@@ -122,7 +122,10 @@ struct b3d_ctx {
     float *d_centre = nullptr;  // [3][16]: two ping-pong centres and one expand scratch
     std::map<std::tuple<int, int, float>, float *> rot_cache;
 
-    // launch shape of the score kernel
+    std::vector<float> obj_z;  // camera depth of each object at b3d_set_scene (see pick_shape)
+
+    // launch shape of the score kernel; until it is set or tuned, launches take pick_shape's
+    bool shape_set = false;
     int tile_w = 64;
     int cta_threads = 256;
     int ctas_per_sm = 0;
@@ -423,6 +426,71 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
     sv.stats = (ctx->instr & B3D_INSTR_WORK) ? ctx->d_stats : nullptr;
     sv.tile_w = ctx->tile_w;
     return sv;
+}
+
+// Launch shape of a score launch (the code of launch_score and the tile width) when none was
+// set or tuned: single calls, each stage of an enumeration and batched launches. Shapes differ
+// in the order of the FP32 sums (1e-8 of a score); a server, whose results must not depend on
+// what shares a batch, fixes one. The CTA size follows the work of a hypothesis, estimated in microseconds of an
+// SM from the slot object's rectangles q and its size D in pixels at the scene's pose:
+//   c = 0.35 + 0.00113 q + D^2 (0.0003 + e (2w+1)^2), e = 0.00006 (ball) or 0.0001 (Gaussian),
+// a fit to a sweep of 33 shapes over 64x48 to 320x240 images, objects of 600 to 12,000 cells
+// and both likelihoods. Up to 1.3 us a hypothesis 32 threads are the fastest (30,000
+// hypotheses of 873 cells at 160x120: 175 us; 64: 205, 128: 236, 256: 398), up to 2.6 64
+// (5,109 cells, 160x120: 453; 128: 463, 256: 696), up to 5.8 128 (17,536 cells,
+// 160x120: 865; 64: 971, 256: 1,094), above 256 with tiles of 128 pixels (320x240: 1,867;
+// 256 threads with 64-pixel tiles 2,337, 128 threads 2,367). A call of few hypotheses takes
+// larger CTAs, so that each SM still has some 600 threads: 1,000 hypotheses of the first
+// object take 15 us with 128 threads, 24 with 256; 300 take 12 with 256, 13 with 64.
+// Calls that kept 256 threads and 64-pixel tiles before: 1,000 hypotheses at 64x48 36 -> 26 us,
+// 16,001 smooth 5x5 ones at 150x113 470 -> 367, 31,250 at 320x240 1,569 -> 1,324, eight scenes
+// batched 721 -> 595, a tracking step at 320x240 370 -> 318.
+struct ScoreShape {
+    int code, tile_w;
+};
+
+double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L) {
+    const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
+    double d2 = 0;
+    for (int k = 0; k < 3; ++k) d2 += (double)(m.hi[k] - m.lo[k]) * (m.hi[k] - m.lo[k]);
+    const double z = std::max((double)ctx->obj_z[slot], 0.5 * std::sqrt(d2) + ctx->cam.near_z);
+    const double f = std::max(ctx->cam.fx, ctx->cam.fy), side = 2.0 * L.w + 1.0;
+    const double px2 = std::min(d2 * f * f / (z * z), (double)ctx->cam.W * ctx->cam.H);
+    return 0.35 + 0.00113 * m.n_quads + px2 * (0.0003 + (L.kind == 0 ? 0.00006 : 0.0001) * side * side);
+}
+
+ScoreShape shape_of_cost(double cost, int64_t n) {
+    const int64_t want = 152 * 600;  // threads that keep the device busy
+    int nt = cost <= 1.3 ? 32 : (cost <= 2.6 ? 64 : (cost <= 5.8 ? 128 : 256));
+    while (nt < 256 && n * nt < want) nt *= 2;
+    const int code = nt == 128 ? 1 : (nt == 64 ? 2 : (nt == 32 ? 3 : 0));
+    return ScoreShape{code << 8, nt == 256 ? 128 : (nt == 128 ? 96 : nt)};
+}
+
+ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, int64_t n) {
+    const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
+    // half windows without a compiled-in scorer and triangle meshes keep the general shape
+    if (ctx->shape_set || m.n_quads <= 0 || L.w < 1 || L.w > 2) return ScoreShape{ctx->score_code(), ctx->tile_w};
+    return shape_of_cost(score_cost(ctx, slot, L), n);
+}
+
+// The shape of one batched launch: of the cost of a hypothesis, weighted by the time its scene
+// takes. slot(i), lik(i) and n(i): scene, slot, likelihood and hypotheses of item i.
+template <class Scene, class Slot, class Hyps>
+ScoreShape pick_shape_multi(const b3d_ctx *owner, int n_items, Scene scene, Slot slot, Hyps hyps, const std::vector<Lik> &Ls) {
+    const ScoreShape set{owner->score_code(), owner->tile_w};
+    if (owner->shape_set) return set;
+    double t = 0, tc = 0;
+    int64_t total = 0;
+    for (int i = 0; i < n_items; ++i) {
+        const b3d_ctx *sc = scene(i);
+        if (sc->meshes[sc->obj_mesh[slot(i)]].n_quads <= 0 || Ls[i].w < 1 || Ls[i].w > 2) return set;
+        const double c = score_cost(sc, slot(i), Ls[i]);
+        t += c * (double)hyps(i);
+        tc += c * c * (double)hyps(i);
+        total += hyps(i);
+    }
+    return t > 0 ? shape_of_cost(tc / t, total) : set;
 }
 
 // A hypothesis counter for one persistent launch (its launcher zeroes it): a ring, so launches
@@ -1143,6 +1211,8 @@ b3d_status b3d_set_scene(b3d_ctx *ctx, const b3d_intrinsics *intr, int32_t n_obj
     c.inv_fx = 1.0f / intr->fx; c.inv_fy = 1.0f / intr->fy;
     ctx->cam = c;
     ctx->obj_mesh.assign(mesh_ids, mesh_ids + n_obj);
+    ctx->obj_z.resize(n_obj);
+    for (int32_t k = 0; k < n_obj; ++k) ctx->obj_z[k] = poses[16 * k + 11];
     ctx->tri_base.assign(n_obj, 0);
     for (int32_t k = 1; k < n_obj; ++k) ctx->tri_base[k] = ctx->tri_base[k - 1] + ctx->meshes[mesh_ids[k - 1]].n_faces;
     {
@@ -1229,7 +1299,9 @@ b3d_status b3d_score_batch(b3d_ctx *ctx, int32_t obj_slot, int64_t n_hyp, const 
         Timed tm(ctx, B3D_K_SCORE, s);
         SceneView sv = scene_view(ctx, obj_slot);
         sv.work = take_work(ctx);
-        launch_score_list(sv, L, PoseList{poses_dev}, n_hyp, loglik_dev, ctx->score_code(), s);
+        const ScoreShape shape = pick_shape(ctx, obj_slot, L, n_hyp);
+        sv.tile_w = shape.tile_w;
+        launch_score_list(sv, L, PoseList{poses_dev}, n_hyp, loglik_dev, shape.code, s);
     }
     ++ctx->launches;
     return check_launch(ctx, "score_batch");
@@ -1463,7 +1535,9 @@ b3d_status b3d_enumerate_c2f(b3d_ctx *ctx, int32_t obj_slot, const float *centre
         P.step = sch->stage[t].step;
         {
             Timed tm(ctx, B3D_K_SCORE, s);
-            launch_score_grid(sv, L, P, n_t[t], ctx->d_ll, ctx->score_code(), s);
+            const ScoreShape shape = pick_shape(ctx, obj_slot, L, n_t[t]);
+            sv.tile_w = shape.tile_w;
+            launch_score_grid(sv, L, P, n_t[t], ctx->d_ll, shape.code, s);
         }
         {
             Timed tm(ctx, B3D_K_RESAMPLE, s);
@@ -1524,6 +1598,9 @@ b3d_status b3d_score_multi(b3d_ctx *owner, int32_t n_items, const b3d_score_item
         const double cb = (double)items[b].n_hyp * items[b].scene->cam.W * items[b].scene->cam.H;
         return ca > cb;
     });
+    const ScoreShape shape = pick_shape_multi(
+        owner, n_items, [&](int i) { return items[i].scene; }, [&](int i) { return items[i].obj_slot; },
+        [&](int i) { return items[i].n_hyp; }, Ls);
     const size_t off_items = 0, off_begin = align16(sizeof(BatchItem) * n_items);
     const size_t bytes = off_begin + align16(sizeof(int64_t) * (n_items + 1));
     unsigned char *h = nullptr;
@@ -1537,7 +1614,7 @@ b3d_status b3d_score_multi(b3d_ctx *owner, int32_t n_items, const b3d_score_item
         BatchItem b;
         memset(&b, 0, sizeof b);
         b.S = scene_view(it.scene, it.obj_slot);
-        b.S.tile_w = owner->tile_w;
+        b.S.tile_w = shape.tile_w;
         b.S.stats = nullptr;
         b.L = Ls[order[k]];
         b.list = PoseList{it.poses_dev};
@@ -1555,7 +1632,7 @@ b3d_status b3d_score_multi(b3d_ctx *owner, int32_t n_items, const b3d_score_item
         cudaMemsetAsync(owner->d_bwork, 0, sizeof(unsigned long long), s);
         launch_score_multi(reinterpret_cast<const BatchItem *>(owner->d_batch + off_items), n_items,
                            reinterpret_cast<const int64_t *>(owner->d_batch + off_begin), total, owner->batch_chunk,
-                           owner->d_bwork, lik->half_window, max_lat, owner->score_code(), s);
+                           owner->d_bwork, lik->half_window, max_lat, shape.code, s);
     }
     ++owner->launches;
     return check_launch(owner, "score_multi");
@@ -1646,13 +1723,17 @@ b3d_status b3d_enumerate_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_it
         macc += items[i].schedule.n_particles;
     }
     std::vector<int64_t> totals(T);
-    std::vector<int> blocks(T);
+    std::vector<int> blocks(T), codes(T);
     for (int t = 0; t < T; ++t) {
         BatchItem *bi = reinterpret_cast<BatchItem *>(h + o_bi) + (size_t)t * n_items;
         LseItem *li = reinterpret_cast<LseItem *>(h + o_li) + (size_t)t * n_items;
         SelectItem *si = reinterpret_cast<SelectItem *>(h + o_si) + (size_t)t * n_items;
         int64_t *ib = reinterpret_cast<int64_t *>(h + o_ib) + (size_t)t * (n_items + 1);
         int *bb = reinterpret_cast<int *>(h + o_bb) + (size_t)t * (n_items + 1);
+        const ScoreShape shape = pick_shape_multi(
+            owner, n_items, [&](int i) { return items[i].scene; }, [&](int i) { return items[i].obj_slot; },
+            [&](int i) { return nh[(size_t)i * T + t]; }, Ls);
+        codes[t] = shape.code;
         int64_t acc = 0;
         int bacc = 0;
         int64_t pacc = 0;
@@ -1671,7 +1752,7 @@ b3d_status b3d_enumerate_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_it
             BatchItem b;
             memset(&b, 0, sizeof b);
             b.S = scene_view(it.scene, it.obj_slot);
-            b.S.tile_w = owner->tile_w;
+            b.S.tile_w = shape.tile_w;
             b.S.stats = nullptr;
             b.L = Ls[i];
             b.grid = P;
@@ -1733,7 +1814,7 @@ b3d_status b3d_enumerate_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_it
             Timed tm(owner, B3D_K_SCORE, s);
             launch_score_multi(reinterpret_cast<const BatchItem *>(d + o_bi) + (size_t)t * n_items, n_items,
                                reinterpret_cast<const int64_t *>(d + o_ib) + (size_t)t * (n_items + 1), totals[t],
-                               owner->batch_chunk, owner->d_bwork + t, lik->half_window, max_lat, owner->score_code(), s);
+                               owner->batch_chunk, owner->d_bwork + t, lik->half_window, max_lat, codes[t], s);
         }
         {
             Timed tm(owner, B3D_K_RESAMPLE, s);
@@ -1858,6 +1939,7 @@ b3d_status b3d_set_tuning(b3d_ctx *ctx, const b3d_tuning *t) {
     if (t->ctas_per_sm < 0 || t->ctas_per_sm > 32) return fail(ctx, B3D_EINVAL, "ctas_per_sm must be in [0, 32]");
     if (t->high_occupancy != 0 && t->high_occupancy != 1) return fail(ctx, B3D_EINVAL, "high_occupancy must be 0 or 1");
     if (t->batch_chunk < 1 || t->batch_chunk > 1024) return fail(ctx, B3D_EINVAL, "batch_chunk must be in [1, 1024]");
+    ctx->shape_set = true;
     ctx->batch_chunk = t->batch_chunk;
     ctx->tile_w = t->tile_w;
     ctx->cta_threads = t->cta_threads;
@@ -1928,6 +2010,7 @@ b3d_status b3d_autotune(b3d_ctx *ctx, int32_t obj_slot, const float *centre_pose
     ctx->cta_threads = win.cta_threads;
     ctx->ctas_per_sm = win.ctas_per_sm;
     ctx->high_occupancy = win.high_occupancy;
+    ctx->shape_set = true;
     if (best) *best = win;
     return check_launch(ctx, "autotune");
 }
@@ -1989,6 +2072,7 @@ b3d_status b3d_autotune_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_ite
         return st;
     }
     apply(win);
+    owner->shape_set = true;
     if (best) *best = win;
     return B3D_OK;
 }
@@ -2076,6 +2160,8 @@ b3d_status b3d_sync(b3d_ctx *ctx, b3d_stream stream) {
 // Context hooks for the tracking server (b3d_server.cu); not part of the C ABI.
 // ==========================================================================================
 namespace b3d {
+
+void ctx_fix_shape(b3d_ctx *ctx) { ctx->shape_set = true; }
 
 uint64_t ctx_used_bytes(b3d_ctx *ctx) { return ctx->used; }
 

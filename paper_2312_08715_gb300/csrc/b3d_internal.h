@@ -268,6 +268,7 @@ void launch_score_noise(const SceneView &sv, const NoiseLik &N, const float *pos
 
 // Context hooks used by the tracking server (defined with the context in b3d_api.cu).
 uint64_t ctx_used_bytes(b3d_ctx *ctx);
+void ctx_fix_shape(b3d_ctx *ctx);  // the score kernel keeps its default launch shape
 void ctx_set_budget(b3d_ctx *ctx, uint64_t budget);
 b3d_status ctx_alloc_bytes(b3d_ctx *ctx, size_t bytes, void **out, const char *what);
 float *ctx_scene_poses(b3d_ctx *ctx);  // device [n_obj, 16]
