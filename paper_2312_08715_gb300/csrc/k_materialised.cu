@@ -21,11 +21,15 @@ namespace b3d {
 // (misses at the far plane) are streamed into the whole image, then the object is drawn by
 // the fused score kernel's renderer (merged voxel rectangles, cooperative raster, 32-bit
 // depth bits) and each tile's composited depths overwrite its fragment box.
-// With triangle ids (k_fill_bg, then k_render_obj): every pixel gets the background key's
-// depth and id (a band of kBandPx background keys stays in shared memory while the CTA
-// streams that band of many images), then the object's triangles over its screen box, with
-// 64-bit atomicMin on packed (depth bits, triangle id) (the nearest fragment wins, equal
-// depths go to the smaller id), overwrite the pixels where they are nearer.
+// With triangle ids (k_render_obj): every pixel gets the background key's depth and id, then
+// the object's triangles over its screen box, with 64-bit atomicMin on packed (depth bits,
+// triangle id) (the nearest fragment wins, equal depths go to the smaller id), overwrite the
+// pixels where they are nearer. The CTA that draws an image also streams its background: the
+// stores (8 bytes a pixel, the bytes the call cannot do without) run beside other CTAs'
+// rasterising, which is bound by instruction issue, instead of in a launch of their own
+// (2,048 images of 160x120: 171 -> 150 us, 321x241: 1,439 -> 1,312; 450 of 160x120: 45 -> 35).
+// Few large images are filled by a launch over all SMs first (k_fill_bg: a band of kBandPx
+// background keys stays in shared memory while the CTA streams that band of the images).
 constexpr int kBandPx = 4096;
 
 inline int n_bands(int64_t npx) { return (int)((npx + kBandPx - 1) / kBandPx); }
@@ -62,7 +66,66 @@ __global__ void __launch_bounds__(256) k_fill_bg(Cam c, const unsigned long long
     }
 }
 
-template <class PS>
+// Pixels of an image of n 4-byte values before its first 16-byte boundary.
+__device__ __forceinline__ int align_head(const void *image, int64_t n) {
+    return (int)min((int64_t)((16u - ((uintptr_t)image & 15u)) & 15u) >> 2, n);
+}
+
+// The background keys' depths and ids into one image, by the CTA. FILL = 4: 16-byte stores
+// between the image's first and last 16-byte boundaries (both outputs at the same offset from
+// one), else 1: pixel by pixel.
+template <int FILL>
+__device__ __forceinline__ void fill_image(const unsigned long long *bg, float *depth, int *tri, int64_t npx, float far_z) {
+    const int tid = threadIdx.x;
+    auto dep = [&](unsigned hi) { return hi == 0xffffffffu ? far_z : __uint_as_float(hi); };
+    // the low word of an empty key is its id, -1
+    auto one = [&](int64_t i) {
+        const unsigned long long key = __ldg(bg + i);
+        __stcs(depth + i, dep((unsigned)(key >> 32)));
+        __stcs(tri + i, (int)(unsigned)key);
+    };
+    if (FILL == 1) {
+        for (int64_t i = tid; i < npx; i += kThreads) one(i);
+        return;
+    }
+    const int head = align_head(depth, npx), n4 = (int)((npx - head) / 4), rest = (int)(npx - head) & 3;
+    if (tid < head + rest) one(tid < head ? tid : npx - rest + (tid - head));  // before and after the vectors
+    float4 *d4 = reinterpret_cast<float4 *>(depth + head);
+    int4 *t4 = reinterpret_cast<int4 *>(tri + head);
+    const unsigned long long *src = bg + head;
+    const bool even = (head & 1) == 0;  // two 8-byte keys to a load
+    auto get = [&](int k, uint4 &a, uint4 &b) {
+        if (even) {
+            a = __ldg(reinterpret_cast<const uint4 *>(src) + 2 * k);
+            b = __ldg(reinterpret_cast<const uint4 *>(src) + 2 * k + 1);
+        } else {
+            const uint2 *p = reinterpret_cast<const uint2 *>(src) + 4 * k;
+            const uint2 u0 = __ldg(p), u1 = __ldg(p + 1), u2 = __ldg(p + 2), u3 = __ldg(p + 3);
+            a = make_uint4(u0.x, u0.y, u1.x, u1.y);
+            b = make_uint4(u2.x, u2.y, u3.x, u3.y);
+        }
+    };
+    auto put = [&](int k, const uint4 &a, const uint4 &b) {
+        __stcs(d4 + k, make_float4(dep(a.y), dep(a.w), dep(b.y), dep(b.w)));
+        __stcs(t4 + k, make_int4((int)a.x, (int)a.z, (int)b.x, (int)b.z));
+    };
+    int k = tid;
+    for (; k + kThreads < n4; k += 2 * kThreads) {  // two vectors' loads in flight (four: slower, registers)
+        uint4 a0, b0, a1, b1;
+        get(k, a0, b0);
+        get(k + kThreads, a1, b1);
+        put(k, a0, b0);
+        put(k + kThreads, a1, b1);
+    }
+    if (k < n4) {
+        uint4 a0, b0;
+        get(k, a0, b0);
+        put(k, a0, b0);
+    }
+}
+
+// FILL: of fill_image; 0: the images hold the background already.
+template <class PS, int FILL>
 __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, int64_t n_hyp, float *out_depth,
                                                          int *out_tid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -83,6 +146,8 @@ __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, i
             __syncwarp();
             tri_view_warp(m, s_pose, c, lane, s_bb, &s_flags, &s_rg);
         }
+        // the barriers below order these stores before the object's
+        if (FILL) fill_image<FILL>(S.bg, out_depth + h * npx, out_tid + h * npx, npx, c.far_z);
         __syncthreads();
         if (!(s_flags & 1)) continue;
         const int bx0 = s_bb[0], bx1 = s_bb[1], by0 = s_bb[2], by1 = s_bb[3];
@@ -113,7 +178,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, i
                         const int64_t gi = (int64_t)(ty0 + y) * c.W + (tx0 + x);
                         if (key < S.bg[gi]) {
                             out_depth[h * npx + gi] = key_depth(key, 0, c.far_z);
-                            if (out_tid) out_tid[h * npx + gi] = (int)(unsigned)(key & 0xffffffffu);
+                            out_tid[h * npx + gi] = (int)(unsigned)(key & 0xffffffffu);
                         }
                     }
                     x += dr;
@@ -457,6 +522,8 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
 // launchers
 // ------------------------------------------------------------------------------------------
 static bool aligned16p(const void *p) { return ((uintptr_t)p & 15u) == 0; }
+// two images of 4-byte values whose 16-byte boundaries fall on the same pixels
+static bool same_offset16(const void *a, const void *b) { return (((uintptr_t)a ^ (uintptr_t)b) & 15u) == 0; }
 
 // persistent grid: as many CTAs as fit (or `grid` when > 0), at most one per item
 template <class K>
@@ -477,20 +544,31 @@ constexpr int kMatNT = 128, kRenderMinB = 8;
 template <int WT>
 constexpr int score_fused_minb(bool whole) { return WT == 1 ? (whole ? 7 : 8) : 6; }
 
+// Renders with ids of fewer than kFillFew images of more than kFillPx pixels fill them in a
+// launch of their own: a CTA needs 10 us to stream an image of 76,800 pixels, the device less
+// than 2 for 16 of them (16 images of 320x240: 90 us, 95 when each CTA fills its own; 150:
+// 121 and 115; 16 of 160x120: 33 and 29).
+constexpr int kFillFew = 100, kFillPx = 40000;
+
 int launch_render_list(const SceneView &sv, PoseList P, int64_t n, float *depth, int *tid, int grid, cudaStream_t s) {
     if (n <= 0) return 0;
     const int64_t npx = (int64_t)sv.cam.W * sv.cam.H;
     if (tid) {
-        const bool vec = npx % 4 == 0 && aligned16p(depth) && aligned16p(tid);
-        auto fill = vec ? k_fill_bg<4> : k_fill_bg<1>;
-        const int nb = n_bands(npx);
-        const int per_sm = kernel_ctas_per_sm(fill, 256, 0);
-        const int64_t x = std::max<int64_t>(1, ((int64_t)per_sm * score_sm_count() + nb - 1) / nb);
-        fill<<<dim3((unsigned)std::min<int64_t>(x, n), (unsigned)nb), 256, 0, s>>>(sv.cam, sv.bg, n, depth, tid);
         const int smem = kRegionPx * (int)sizeof(unsigned long long);
-        auto kern = k_render_obj<PoseList>;
+        if (n < kFillFew && npx > kFillPx) {
+            const bool vec = npx % 4 == 0 && aligned16p(depth) && aligned16p(tid);
+            auto fill = vec ? k_fill_bg<4> : k_fill_bg<1>;
+            const int nb = n_bands(npx);
+            const int per_sm = kernel_ctas_per_sm(fill, 256, 0);
+            const int64_t x = std::max<int64_t>(1, ((int64_t)per_sm * score_sm_count() + nb - 1) / nb);
+            fill<<<dim3((unsigned)std::min<int64_t>(x, n), (unsigned)nb), 256, 0, s>>>(sv.cam, sv.bg, n, depth, tid);
+            auto kern = k_render_obj<PoseList, 0>;
+            kern<<<persistent_grid(kern, kThreads, smem, n, grid), kThreads, smem, s>>>(sv, P, n, depth, tid);
+            return 2;
+        }
+        auto kern = same_offset16(depth, tid) ? k_render_obj<PoseList, 4> : k_render_obj<PoseList, 1>;
         kern<<<persistent_grid(kern, kThreads, smem, n, grid), kThreads, smem, s>>>(sv, P, n, depth, tid);
-        return 2;
+        return 1;
     }
     const bool vec = npx % 4 == 0 && aligned16p(depth);
     const int n_lat = sv.mesh.nc[0] + sv.mesh.nc[1] + sv.mesh.nc[2];
