@@ -191,9 +191,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, i
     }
 }
 
-// V = 4: 16-byte vector accesses (the image size a multiple of 4 pixels and the buffers
-// 16-byte aligned), else 1.
-template <int NT, int MINB, int V>
+template <int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB) k_render_fused(SceneView S, PoseList P, int64_t n_hyp, float *out_depth) {
     constexpr int REG = score_region<NT>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -216,19 +214,32 @@ __global__ void __launch_bounds__(NT, MINB) k_render_fused(SceneView S, PoseList
         }
         float *dst = out_depth + h * npx;
         // the background first; render_tiles' barriers order these stores before the tiles'
-        if (V == 4) {  // four loads in flight per thread
-            const float4 *src = reinterpret_cast<const float4 *>(S.bgd);
-            float4 *d4 = reinterpret_cast<float4 *>(dst);
-            const int n4 = (int)(npx / 4);
-            int k = tid;
-            for (; k + 3 * NT < n4; k += 4 * NT) {
-                const float4 a0 = __ldg(src + k), a1 = __ldg(src + k + NT), a2 = __ldg(src + k + 2 * NT),
-                             a3 = __ldg(src + k + 3 * NT);
-                __stcs(d4 + k, a0); __stcs(d4 + k + NT, a1); __stcs(d4 + k + 2 * NT, a2); __stcs(d4 + k + 3 * NT, a3);
+        {  // 16-byte stores between the image's 16-byte boundaries, four loads in flight per thread.
+            // An image of 161x121 starts at any offset from one: pixel by pixel its stores held
+            // the CTA up (10,000 images, rendered and scored: 564 us against 433 for 160x120; now
+            // 480 and 422)
+            const int head = align_head(dst, npx);
+            const int n4 = (int)((npx - head) / 4), rest = (int)(npx - head) & 3;
+            float4 *d4 = reinterpret_cast<float4 *>(dst + head);
+            auto stream = [&](auto get) {
+                int k = tid;
+                for (; k + 3 * NT < n4; k += 4 * NT) {
+                    const float4 a0 = get(k), a1 = get(k + NT), a2 = get(k + 2 * NT), a3 = get(k + 3 * NT);
+                    __stcs(d4 + k, a0); __stcs(d4 + k + NT, a1); __stcs(d4 + k + 2 * NT, a2); __stcs(d4 + k + 3 * NT, a3);
+                }
+                for (; k < n4; k += NT) __stcs(d4 + k, get(k));
+            };
+            if (head == 0) {
+                stream([&](int k) { return __ldg(reinterpret_cast<const float4 *>(S.bgd) + k); });
+            } else {
+                const float *src = S.bgd + head;
+                stream([&](int k) {
+                    const float *p = src + 4 * k;
+                    return make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+                });
+                if (tid < head) dst[tid] = __ldg(S.bgd + tid);
             }
-            for (; k < n4; k += NT) __stcs(d4 + k, __ldg(src + k));
-        } else {
-            for (int64_t k = tid; k < npx; k += NT) __stcs(dst + k, __ldg(S.bgd + k));
+            if (tid < rest) dst[npx - rest + tid] = __ldg(S.bgd + (npx - rest + tid));
         }
         render_tiles<false, NT>(S, 0, 0, sh, s_stage, zb, lat, nullptr,
                                 [&](const float *zd, int zx0, int zy0, int zw, int qx0, int qx1, int qy0, int qy1, int, int, int, int) {
@@ -262,7 +273,8 @@ __global__ void __launch_bounds__(NT, MINB) k_render_fused(SceneView S, PoseList
 //     read back through the cache, tile by tile in shared memory), with the sliding-window
 //     column scorer of the fused kernel (WT = 1, 2) or pixel_ell (WT = 0):
 //       LL_h = LL_bg + sum_{i in box + w} (l_i - l_i(bg)).
-// MM = 1: miss mode 1 (pixels with id -1 carry no point).
+// MM = 1: miss mode 1 (pixels with id -1 carry no point). V = 4: step 1 reads 16-byte vectors
+// between the image's 16-byte boundaries (with MM the ids' too), else 1: pixel by pixel.
 __device__ __forceinline__ void box_note(int i, int W, int &x0, int &x1, int &y0, int &y1) {
     const int y = i / W, x = i - y * W;
     x0 = min(x0, x); x1 = max(x1, x); y0 = min(y0, y); y1 = max(y1, y);
@@ -313,9 +325,12 @@ __device__ __forceinline__ float score_column_ball3(const SceneView &S, const Li
     load(pa, sa, na);
     load(pb, sb, nb);
     float acc = 0.f;
+    int left = yb - ya + 1;
+    float2 next = *qp;  // the row's inputs are loaded a row ahead of their use
     auto score = [&](float nmid) {
-        const float2 qe = *qp;  // observed depth (0: no point) and the background's term
+        const float2 qe = next;  // observed depth (0: no point) and the background's term
         qp += c.W;
+        if (--left > 0) next = *qp;
         // the observed point, formed from its depth as the observation kernel forms it
         const float qx = __fmul_rn(qe.x, rx1), qy = __fmul_rn(qe.x, -nmid);
         const f32x2_t qx2 = pk2(qx, qx), qy2 = pk2(qy, qy), qz2 = pk2(qe.x, qe.x);
@@ -337,16 +352,16 @@ __device__ __forceinline__ float score_column_ball3(const SceneView &S, const Li
         const float l = lut[__float_as_int(nf) & 15];
         if (qe.x != 0.f) acc += l - qe.y;
     };
-    for (int left = yb - ya + 1;;) {
+    for (;;) {
         load(pc, sc, nc);
         score(nb);
-        if (--left == 0) break;
+        if (left == 0) break;
         load(pa, sa, na);
         score(nc);
-        if (--left == 0) break;
+        if (left == 0) break;
         load(pb, sb, nb);
         score(na);
-        if (--left == 0) break;
+        if (left == 0) break;
     }
     return acc;
 }
@@ -401,31 +416,41 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
         if (whole) {
             x0 = 0; x1 = c.W - 1; y0 = 0; y1 = c.H - 1;
         } else if (V == 4) {
-            const int64_t n4 = npx / 4;
-            const float4 *src = reinterpret_cast<const float4 *>(img);
-            const int4 *tsrc = reinterpret_cast<const int4 *>(tim);
-            const float4 *gsrc = reinterpret_cast<const float4 *>(bgd);
-            for (int64_t k0 = tid; k0 < n4; k0 += U * NT) {
+            const int head = align_head(img, npx), n4 = (int)((npx - head) / 4), rest = (int)(npx - head) & 3;
+            const float4 *src = reinterpret_cast<const float4 *>(img + head);
+            const int4 *tsrc = reinterpret_cast<const int4 *>(MM ? tim + head : nullptr);
+            const float *gsrc = bgd + head;
+            const bool galigned = ((uintptr_t)gsrc & 15u) == 0;
+            auto get_g = [&](int k) {
+                const float *p = gsrc + 4 * k;
+                return galigned ? __ldg(reinterpret_cast<const float4 *>(p))
+                                : make_float4(__ldg(p), __ldg(p + 1), __ldg(p + 2), __ldg(p + 3));
+            };
+            if (tid < head + rest) {  // the pixels before and after the vectors
+                const int i = tid < head ? tid : (int)npx - rest + (tid - head);
+                if (differs(i)) box_note(i, c.W, x0, x1, y0, y1);
+            }
+            for (int k0 = tid; k0 < n4; k0 += U * NT) {
                 float4 d[U], g[U];
                 int4 t[U];
 #pragma unroll
                 for (int j = 0; j < U; ++j) {
-                    const int64_t k = k0 + j * NT;
+                    const int k = k0 + j * NT;
                     const bool ok = k < n4;
                     d[j] = ok ? __ldg(src + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-                    g[j] = ok ? __ldg(gsrc + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    g[j] = ok ? get_g(k) : make_float4(0.f, 0.f, 0.f, 0.f);
                     t[j] = (MM && ok) ? __ldg(tsrc + k) : make_int4(0, 0, 0, 0);
                 }
 #pragma unroll
                 for (int j = 0; j < U; ++j) {
-                    const int64_t k = k0 + j * NT;
+                    const int k = k0 + j * NT;
                     const float e[4] = {t[j].x < 0 ? -1.f : d[j].x, t[j].y < 0 ? -1.f : d[j].y,
                                         t[j].z < 0 ? -1.f : d[j].z, t[j].w < 0 ? -1.f : d[j].w};
                     const float b[4] = {g[j].x, g[j].y, g[j].z, g[j].w};
                     unsigned mask = 0;
 #pragma unroll
                     for (int v = 0; v < 4; ++v) mask |= __float_as_uint(e[v]) != __float_as_uint(b[v]) ? 1u << v : 0u;
-                    if (mask) box_note4((int)(4 * k), mask, c.W, x0, x1, y0, y1);
+                    if (mask) box_note4(head + 4 * k, mask, c.W, x0, x1, y0, y1);
                 }
             }
         } else {
@@ -462,14 +487,23 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                     {
                         const int dq = NT / zw, dr = NT - dq * zw;
                         int y = tid / zw, x = tid - y * zw;
-                        for (int i = tid; i < nz; i += NT) {
-                            const int gi = (zy0 + y) * c.W + (zx0 + x);  // an image has at most 2^26 pixels
-                            float d = img[gi];
-                            if (MM && tim[gi] < 0) d = -1.f;
-                            zd[i] = d;
-                            x += dr;
-                            y += dq;
-                            if (x >= zw) { x -= zw; ++y; }
+                        for (int i = tid; i < nz; i += U * NT) {
+                            float d[U];
+#pragma unroll
+                            for (int u = 0; u < U; ++u) {
+                                d[u] = 0.f;
+                                if (i + u * NT < nz) {
+                                    const int gi = (zy0 + y) * c.W + (zx0 + x);  // an image has at most 2^26 pixels
+                                    d[u] = __ldg(img + gi);
+                                    if (MM && __ldg(tim + gi) < 0) d[u] = -1.f;
+                                }
+                                x += dr;
+                                y += dq;
+                                if (x >= zw) { x -= zw; ++y; }
+                            }
+#pragma unroll
+                            for (int u = 0; u < U; ++u)
+                                if (i + u * NT < nz) zd[i + u * NT] = d[u];
                         }
                     }
                     __syncthreads();
@@ -570,10 +604,9 @@ int launch_render_list(const SceneView &sv, PoseList P, int64_t n, float *depth,
         kern<<<persistent_grid(kern, kThreads, smem, n, grid), kThreads, smem, s>>>(sv, P, n, depth, tid);
         return 1;
     }
-    const bool vec = npx % 4 == 0 && aligned16p(depth);
     const int n_lat = sv.mesh.nc[0] + sv.mesh.nc[1] + sv.mesh.nc[2];
     const int smem = score_region<kMatNT>() * (int)sizeof(unsigned) + n_lat * (int)sizeof(float4);
-    auto kern = vec ? k_render_fused<kMatNT, kRenderMinB, 4> : k_render_fused<kMatNT, kRenderMinB, 1>;
+    auto kern = k_render_fused<kMatNT, kRenderMinB>;
     if (sv.work) cudaMemsetAsync(sv.work, 0, sizeof(unsigned long long), s);
     kern<<<persistent_grid(kern, kMatNT, smem, n, grid), kMatNT, smem, s>>>(sv, P, n, depth);
     return 1;
@@ -582,12 +615,10 @@ int launch_render_list(const SceneView &sv, PoseList P, int64_t n, float *depth,
 template <int WT, bool WHOLE>
 static void launch_score_fused(const SceneView &sv, const Lik &L, const float *depth, const int *tid, int64_t n,
                                float *ll, int grid, cudaStream_t s) {
-    const int64_t npx = (int64_t)sv.cam.W * sv.cam.H;
     const bool mm = L.miss_mode == 1;
-    const bool vec = npx % 4 == 0 && aligned16p(depth) && (!mm || aligned16p(tid));
     constexpr int MB = score_fused_minb<WT>(WHOLE);
-    auto kern = vec ? (mm ? k_score_fused<WT, kMatNT, MB, 4, 1> : k_score_fused<WT, kMatNT, MB, 4, 0>)
-                    : (mm ? k_score_fused<WT, kMatNT, MB, 1, 1> : k_score_fused<WT, kMatNT, MB, 1, 0>);
+    auto kern = !mm ? k_score_fused<WT, kMatNT, MB, 4, 0>
+                    : (same_offset16(depth, tid) ? k_score_fused<WT, kMatNT, MB, 4, 1> : k_score_fused<WT, kMatNT, MB, 1, 1>);
     if (sv.work) cudaMemsetAsync(sv.work, 0, sizeof(unsigned long long), s);
     kern<<<persistent_grid(kern, kMatNT, 0, n, grid), kMatNT, 0, s>>>(sv, L, depth, tid, n, ll);
 }

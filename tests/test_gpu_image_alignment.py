@@ -67,3 +67,47 @@ def test_few_and_many_large_images(orc):
     ctx.sync()
     assert all(torch.equal(a[:99], b) for a, b in zip(many, few))
     ctx.close()
+
+
+@pytest.mark.parametrize("width,height", SIZES)
+def test_depth_renders_and_scores(orc, width, height):
+    """The depth render is the same bits at every offset and writes nothing around the images;
+    its scores, and those of images changed at their first and last pixels, are the same bits at
+    every offset and within 1e-4 of the summed |l_i| of the oracle's per-pixel terms."""
+    from paper_2312_08715_gb300 import b3d
+    wl, ctx, P = _scene(orc, width, height, 5)
+    Pd = torch.as_tensor(P, device="cuda")
+    n = len(P) * width * height
+    obs = observed(orc, wl)
+    rng = np.random.default_rng(7)
+    first = ids = None
+    for off in range(4):
+        bd, d = _buffer(n, off, torch.float32)
+        b3d.b3d_render_batch(ctx.h, wl.slot, len(P), Pd, d, None, ctx.stream)
+        ctx.sync()
+        assert _untouched(bd, off, n)
+        if first is None:
+            first = d.clone()
+            ids = torch.as_tensor(np.where(rng.random(n) < 0.2, -1, 3).astype(np.int32), device="cuda")
+        assert torch.equal(d, first), off
+    imgs = first.clone().reshape(len(P), -1)
+    imgs[1:, 0] += 0.05
+    imgs[2:, -1] -= 0.05
+    for half_window in (1, 2):
+        for miss_mode in (0, 1):
+            lk = dict(kind=0, radius=0.005, p_outlier=0.01, half_window=half_window, miss_mode=miss_mode)
+            got = []
+            for od, ot in [(0, 0), (1, 1), (2, 2), (3, 3), (0, 3), (2, 1)]:
+                (_, d), (_, t) = _buffer(n, od, torch.float32), _buffer(n, ot, torch.int32)
+                d.copy_(imgs.reshape(-1))
+                t.copy_(ids)
+                shape = (len(P), height, width)
+                got.append(ctx.score_depth(d.view(shape), lk, t.view(shape) if miss_mode else None, slot=wl.slot))
+            ctx.sync()
+            assert all(torch.equal(g, got[0]) for g in got)
+            for k in range(len(P)):
+                im = imgs[k].reshape(height, width).cpu().numpy().astype(np.float64)
+                i = ids.reshape(len(P), height, width)[k].cpu().numpy() if miss_mode else None
+                ell = orc.pixel_loglik(wl.scene.camera, lk, im, i, obs)[0]
+                assert abs(float(got[0][k]) - ell.sum()) <= 1e-4 * np.abs(ell).sum()
+    ctx.close()
