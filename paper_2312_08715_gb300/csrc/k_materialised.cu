@@ -164,7 +164,7 @@ __global__ void __launch_bounds__(kThreads, 3) k_render_obj(SceneView S, PS P, i
                     atomicMin(&zb[(y - ty0) * zw + (x - tx0)], pack_key(z, gid));
                 };
                 for (int base = wid * 32; base < s_rg.total; base += nt)
-                    tri_batch(m, s_rg, s_flags, s_pose, S.tri_base, c, base, tx0, tx1, ty0, ty1, &s_hq, store);
+                    tri_batch(m, s_rg, s_flags, s_pose, S.tri_base, c, base, 32, tx0, tx1, ty0, ty1, &s_hq, store);
                 __syncthreads();
                 if (s_hq.n > 0) {
                     tri_huge<kThreads>(s_hq, c, store);

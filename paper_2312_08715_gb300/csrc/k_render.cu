@@ -36,17 +36,27 @@ struct CamObject {
     float pose[12];
     int bb[4];
     int flags;
+    int shift;  // log2 of the triangles a batch holds
     TriRanges rg;
 };
+
+// Objects of kCamLarge pixels of screen box a triangle and more go out 8 triangles to a batch
+// in CTAs of more than 8 warps: a warp tests such triangles one after another, and 32 of an
+// 800-triangle table were a warp's whole share of a hypothesis, at whose end the others waited
+// (2,048 hypotheses at 200x200: 1,154 -> 905 us). With 24 as the line, or with 8 warps a CTA,
+// the set-up of 8 lanes costs more than it evens out (1,500 hypotheses of 150x150 867 -> 872
+// us, of 100x100 353 -> 357).
+constexpr float kCamLarge = 40.f;
 
 // Order of n objects by pixels of screen box per triangle, largest first (ties by index), by
 // one warp (n <= 32): batches of large triangles are handed out first, so the last batches of
 // a hypothesis are short ones (a table's batch costs 20 times a voxel mesh's).
-__device__ __forceinline__ void cam_order_warp(const CamObject *obj, int n, int lane, int *order) {
+__device__ __forceinline__ void cam_order_warp(CamObject *obj, int n, int lane, int nt, int *order) {
     float key = -1.f;
     if (lane < n && (obj[lane].flags & 1)) {
         const int *bb = obj[lane].bb;
         key = (float)(bb[1] - bb[0] + 1) * (float)(bb[3] - bb[2] + 1) / (float)max(obj[lane].rg.total, 1);
+        obj[lane].shift = nt > 256 && key >= kCamLarge ? 3 : 5;
     }
     int rank = 0;
     for (int j = 0; j < n; ++j) {
@@ -85,7 +95,7 @@ __device__ __forceinline__ void cam_raster(const CamObject *obj, const int *orde
         b = __shfl_sync(0xffffffffu, b, 0);
         while (i < n) {
             const CamObject &o = obj[order[i]];
-            const int nb = (o.flags & 1) ? (o.rg.total + 31) >> 5 : 0;
+            const int sh = NT > 256 ? o.shift : 5, nb = (o.flags & 1) ? (o.rg.total + (1 << sh) - 1) >> sh : 0;
             if (b < before + nb) break;
             before += nb;
             ++i;
@@ -93,10 +103,11 @@ __device__ __forceinline__ void cam_raster(const CamObject *obj, const int *orde
         if (i >= n) break;
         const int k = order[i];
         const CamObject &o = obj[k];
+        const int sh = NT > 256 ? o.shift : 5;
         const int x0 = max(rx0, o.bb[0]), x1 = min(rx1, o.bb[1]), y0 = max(ry0, o.bb[2]), y1 = min(ry1, o.bb[3]);
         if (x0 > x1 || y0 > y1) continue;
-        tri_batch(meshes[k], o.rg, o.flags, o.pose, tri_base ? tri_base[k] : 0, c, (b - before) << 5, x0, x1, y0, y1, &hq,
-                  store);
+        tri_batch(meshes[k], o.rg, o.flags, o.pose, tri_base ? tri_base[k] : 0, c, (b - before) << sh,
+                  1 << sh, x0, x1, y0, y1, &hq, store);
     }
     __syncthreads();
     tri_huge<NT>(hq, c, store);
@@ -132,7 +143,7 @@ __global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshVie
                     if (n_obj > kMaxCamObjects || (ty0 == 0 && tx0 == 0)) {
                         for (int k = wid; k < n; k += nw) cam_object_warp(s_obj[k], meshes[k0 + k], world + 16 * (k0 + k), P, h, c, lane);
                         __syncthreads();
-                        if (wid == 0) cam_order_warp(s_obj, n, lane, s_order);
+                        if (wid == 0) cam_order_warp(s_obj, n, lane, kThreads, s_order);
                     }
                     if (tid == 0) { s_next = 0; s_hq.n = 0; }
                     __syncthreads();
@@ -173,7 +184,7 @@ __global__ void __launch_bounds__(NT) k_render_camera_depth(Cam c, const MeshVie
     for (int64_t h = blockIdx.x; h < n_hyp; h += gridDim.x) {
         for (int k = wid; k < n_obj; k += NT / 32) cam_object_warp(s_obj[k], meshes[k], world + 16 * k, P, h, c, lane);
         __syncthreads();
-        if (wid == 0) cam_order_warp(s_obj, n_obj, lane, s_order);
+        if (wid == 0) cam_order_warp(s_obj, n_obj, lane, NT, s_order);
         if (tid == 0) { s_next = 0; s_hq.n = 0; }
         __syncthreads();
         cam_raster<NT>(s_obj, s_order, n_obj, meshes, nullptr, c, 0, c.W - 1, 0, c.H - 1, &s_next, s_hq,

@@ -183,17 +183,17 @@ struct HugeQueue {
     int n;
 };
 
-// 32 triangles [base, base + 32) of the ranges, by one warp (all lanes call it).
+// Triangles [base, base + cnt) of the ranges, cnt at most 32, by one warp (all lanes call it).
 template <class Store>
 __device__ __forceinline__ void tri_batch(const MeshView &m, const TriRanges &rg, int flags, const float *pose, int tri_base,
-                                          const Cam &c, int base, int rx0, int rx1, int ry0, int ry1, HugeQueue *hq,
+                                          const Cam &c, int base, int cnt, int rx0, int rx1, int ry0, int ry1, HugeQueue *hq,
                                           Store &&store) {
     const int lane = threadIdx.x & 31;
     const bool front = (flags & 4) != 0;
     const int k = base + lane;
     TriRec T;
     T.n = 0;
-    if (k < rg.total) {
+    if (lane < cnt && k < rg.total) {
         int cls = 0;
 #pragma unroll
         for (int j = 1; j < 6; ++j) cls += k >= rg.pre[j] ? 1 : 0;
