@@ -92,6 +92,18 @@ __device__ __forceinline__ f32x2_t mul2(f32x2_t a, f32x2_t b) {
     return d;
 }
 
+// Smallest of three and of two numbers; NaN if any is NaN.
+__device__ __forceinline__ float min3_nan(float a, float b, float c) {
+    float m;
+    asm("min.NaN.f32 %0, %1, %2, %3;" : "=f"(m) : "f"(a), "f"(b), "f"(c));
+    return m;
+}
+__device__ __forceinline__ float min2_nan(float a, float b) {
+    float m;
+    asm("min.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+    return m;
+}
+
 // Sum of l_i - l_i(bg) over pixel column x, rows [ya, yb], with the (2W+1)^2 window of
 // rendered depths slid down the column in registers. Window slots outside the image (and
 // pixels without a point) hold -1 and contribute nothing; the terms are formed in the same
@@ -216,7 +228,7 @@ constexpr int score_region() { return NT <= 64 ? 2048 : (NT == 128 ? 3072 : 8192
 #define B3D_COMPOSITE_BATCH 4
 #endif
 constexpr int kCompBatch = B3D_COMPOSITE_BATCH;
-constexpr int kStageStride = 6;  // float4 per staged rectangle: four edges, plane, pixel box
+constexpr int kStageStride = 6;  // float4 per staged rectangle: x, y, dx, -dy of its four edges, plane, pixel box
 // Layout of a warp's 32 staged records: component k of lane l's record at [k * 32 + l], so
 // the lanes' stores and the owners' loads touch consecutive 16-byte words (rather than
 // words 96 bytes apart, which shared four banks between lanes l and l + 4).
@@ -230,10 +242,6 @@ __device__ __forceinline__ int stage_slot(int l, int k) { return k * 32 + l; }
 #define B3D_CAND_Y 1
 #endif
 constexpr int kCandX = B3D_CAND_X, kCandY = B3D_CAND_Y;
-
-__device__ __forceinline__ bool staged_inside(const float4 &E, float px, float py) {
-    return fmaf(E.z, py - E.y, -(E.w * (px - E.x))) >= 0.f;
-}
 
 // The mesh's lattice plane coordinates into the .w of the CTA's lattice table, once per
 // mesh (before the barrier that precedes the first render_tiles): each hypothesis's lattice
@@ -406,20 +414,32 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
                     // Each warp takes 32 rectangles at a time: every lane projects one and
                     // stages its screen corners, plane and pixel box; then the warp shares out
                     // the pixel-centre candidates of all 32 among its lanes.
-                    // Candidate block (x, y) of a rectangle with edges E0-E3, plane Pl and pixel
-                    // box ending at (xe, ye):
-                    auto raster_block = [&](const float4 &E0, const float4 &E1, const float4 &E2, const float4 &E3,
+                    // Candidate block (x, y) of a rectangle with edge origins (EX, EY), directions
+                    // (EZ, -EW) (component e: edge e), plane Pl and pixel box ending at (xe, ye).
+                    // The edges are taken two at a time in packed arithmetic, each lane rounded as
+                    // fmaf(dx, py - y, -(dy (px - x))); a record's components are staged by kind so
+                    // that the loaded registers are the packed operands, and the four signs are
+                    // tested as one minimum: 3.5% fewer instructions (145,800 hypotheses at
+                    // 160x120 2,739 -> 2,694 us, 31,250 at 320x240 1,302 -> 1,290).
+                    auto raster_block = [&](const float4 &EX, const float4 &EY, const float4 &EZ, const float4 &EW,
                                             const float4 &Pl, int x, int y, int xe, int ye, bool valid, unsigned tag) {
+                        const f32x2_t ex01 = pk2(EX.x, EX.y), ex23 = pk2(EX.z, EX.w), ey01 = pk2(EY.x, EY.y), ey23 = pk2(EY.z, EY.w);
+                        const f32x2_t ez01 = pk2(EZ.x, EZ.y), ez23 = pk2(EZ.z, EZ.w), ew01 = pk2(EW.x, EW.y), ew23 = pk2(EW.z, EW.w);
 #pragma unroll
                         for (int e = 0; e < kCandY; ++e) {
                             const float py = (float)(y + e) + 0.5f;
+                            const f32x2_t py2 = pk2(py, py);
+                            const f32x2_t v01 = sub2(py2, ey01), v23 = sub2(py2, ey23);
 #pragma unroll
                             for (int d = 0; d < kCandX; ++d) {
                                 const float px = (float)(x + d) + 0.5f;
+                                const f32x2_t px2 = pk2(px, px);
+                                float e0, e1, e2, e3;
+                                upk2(fma2(ez01, v01, mul2(ew01, sub2(px2, ex01))), e0, e1);
+                                upk2(fma2(ez23, v23, mul2(ew23, sub2(px2, ex23))), e2, e3);
                                 // every test evaluated and one predicated store: branches on the
                                 // tests cost more than the tests (the lanes' pixels diverge)
-                                const bool in = valid & (x + d <= xe) & (kCandY == 1 || y + e <= ye) & staged_inside(E0, px, py) &
-                                                staged_inside(E1, px, py) & staged_inside(E2, px, py) & staged_inside(E3, px, py);
+                                const bool in = valid & (x + d <= xe) & (kCandY == 1 || y + e <= ye) & (min2_nan(min3_nan(e0, e1, e2), e3) >= 0.f);
                                 const float z = __fdividef(1.0f, fmaf(Pl.x, px, fmaf(Pl.y, py, Pl.z)));
                                 if (in & (z <= c.far_z)) {
                                     if (STATS) ++cnt[4];
@@ -494,10 +514,10 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
                                     // quotient is at least 1/(2 bw2) from an integer; the error is below
                                     // (k + 1/2) 2^-21 / bw2)
                                     const float4 Pl = make_float4(al, be, K, __fdividef(1.0f, (float)bw2));
-                                    stg[stage_slot(lane, 0)] = E0;
-                                    stg[stage_slot(lane, 1)] = E1;
-                                    stg[stage_slot(lane, 2)] = E2;
-                                    stg[stage_slot(lane, 3)] = E3;
+                                    stg[stage_slot(lane, 0)] = make_float4(E0.x, E1.x, E2.x, E3.x);
+                                    stg[stage_slot(lane, 1)] = make_float4(E0.y, E1.y, E2.y, E3.y);
+                                    stg[stage_slot(lane, 2)] = make_float4(E0.z, E1.z, E2.z, E3.z);
+                                    stg[stage_slot(lane, 3)] = make_float4(-E0.w, -E1.w, -E2.w, -E3.w);
                                     stg[stage_slot(lane, 4)] = Pl;
                                     // box extents below 2^16 and 2^13; TAGS: the class in the top bits
                                     const int ends = (x1 - x0) | ((y1 - y0) << 16) | (TAGS ? cls << 29 : 0);
