@@ -107,12 +107,23 @@ __device__ __forceinline__ float min2_nan(float a, float b) {
     return m;
 }
 
+// Squared distances of an observed point (qx, qy, qz) to two rendered points of depths z on the
+// negated rays (nrx, nry).
+__device__ __forceinline__ f32x2_t dist2(f32x2_t z, f32x2_t nrx, f32x2_t nry, f32x2_t qx, f32x2_t qy, f32x2_t qz) {
+    const f32x2_t ex = fma2(z, nrx, qx), ey = fma2(z, nry, qy), ez = sub2(qz, z);
+    return fma2(ex, ex, fma2(ey, ey, mul2(ez, ez)));
+}
+
 // Sum of l_i - l_i(bg) over pixel column x, rows [ya, yb], with the (2W+1)^2 window of
 // rendered depths slid down the column in registers. Window slots outside the image (and
 // pixels without a point) hold -1 and contribute nothing; the terms are formed in the same
 // order and by the same expressions as pixel_ell, so unchanged pixels give 0 exactly.
-template <int W>
-__device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
+// KIND: L.kind compiled in. The window's elements are taken in packed pairs, Gaussian or ball
+// (PAIRS = false: the 5x5 ball one by one): issue-bound, so a pair saves 7 of its 14 FP32
+// instructions (GB300, us: 20,000 hypotheses at 160x120, Gaussian 5x5 874 -> 765, 3x3 468 ->
+// 440; ball 5x5 563 -> 552; 16,001 Gaussian 5x5 at 150x113 377 -> 333).
+template <int W, int KIND, bool PAIRS = true>
+__device__ __forceinline__ float score_column_kind(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
                                               const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb,
                                               unsigned long long *n_px, unsigned long long *n_pairs) {
     constexpr int D = 2 * W + 1;
@@ -138,8 +149,11 @@ __device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, 
     const bool ball_skips_empty = L.r2 < 0.25f;
     const float r2b = __int_as_float(__float_as_int(L.r2) + 1) * 0x1p100f;  // (next float above r2) 2^100
     const float rxc = rx[W];  // the column's own ray
-    // negated column rays packed for the f32x2 window terms (half window 1)
-    const f32x2_t nrx01 = pk2(-rx[0], -rx[1]), nrx22 = pk2(-rx[D - 1], -rx[D - 1]);
+    // negated column rays packed for the window terms
+    f32x2_t nrx2[W > 0 ? W : 1];
+#pragma unroll
+    for (int k = 0; k < W; ++k) nrx2[k] = pk2(-rx[2 * k], -rx[2 * k + 1]);
+    const f32x2_t nrxl = pk2(-rx[D - 1], -rx[D - 1]);
     for (int y = ya; y <= yb; ++y) {
 #pragma unroll
         for (int r = 0; r + 1 < D; ++r) {
@@ -155,44 +169,72 @@ __device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, 
         const float4 q = make_float4(__fmul_rn(qe.x, rxc), __fmul_rn(qe.x, ry[W]), qe.x, 1.f);
         int n = 0;
         float Ssum = 0.f;
-        if (L.kind == 0 && ball_skips_empty) {
+        if (KIND == 0 && ball_skips_empty) {
             // an empty slot holds z = -1, a point at least 1 m from q (q.z > 0): it can only
             // fail the inlier test, so the count needs no separate z >= 0 test
             // the count on the FMA pipe rather than the (half-rate) ALU pipe: (r2+ - d2) 2^100,
             // saturated to [0, 1], is 1 exactly when d2 <= r2 (r2+ the next float above r2, and
             // any nonzero difference times 2^100 is above 1) and 0 otherwise; the same n as the
             // comparison pixel_ell makes
+            // The window elements in packed pairs: columns 2k, 2k + 1 of each row and the last
+            // column of rows 2k, 2k + 1, the last element scalar: per element the arithmetic of
+            // the loop below, and the 0/1 terms add up exactly in any order
             float nf = 0.f;
-            if constexpr (W == 1) {
-                // eight of the nine window elements as four packed pairs (columns 0-1 of each
-                // row, and column 2 of rows 0-1), the last one scalar: per element the same
-                // arithmetic as the scalar loop below; the 0/1 terms add up exactly in any order
-                const f32x2_t qx2 = pk2(q.x, q.x), qy2 = pk2(q.y, q.y), qz2 = pk2(q.z, q.z);
-                auto pair = [&](f32x2_t z2, f32x2_t nrx, f32x2_t nry) {
-                    const f32x2_t ex = fma2(z2, nrx, qx2), ey = fma2(z2, nry, qy2), ez = sub2(qz2, z2);
-                    float d2a, d2b;
-                    upk2(fma2(ex, ex, fma2(ey, ey, mul2(ez, ez))), d2a, d2b);
-                    nf += __saturatef(fmaf(-d2a, 0x1p100f, r2b));
-                    nf += __saturatef(fmaf(-d2b, 0x1p100f, r2b));
-                };
+            const f32x2_t qx2 = pk2(q.x, q.x), qy2 = pk2(q.y, q.y), qz2 = pk2(q.z, q.z);
+            auto pair = [&](f32x2_t z2, f32x2_t nrx, f32x2_t nry) {
+                float d2a, d2b;
+                upk2(dist2(z2, nrx, nry, qx2, qy2, qz2), d2a, d2b);
+                nf += __saturatef(fmaf(-d2a, 0x1p100f, r2b));
+                nf += __saturatef(fmaf(-d2b, 0x1p100f, r2b));
+            };
+            auto one = [&](int r, int d) {
+                const float z = win[r][d];
+                const float ex = fmaf(-z, rx[d], q.x), ey = fmaf(-z, ry[r], q.y), ez = q.z - z;
+                nf += __saturatef(fmaf(-fmaf(ex, ex, fmaf(ey, ey, ez * ez)), 0x1p100f, r2b));
+            };
+            if constexpr (W == 1 || PAIRS) {
 #pragma unroll
-                for (int r = 0; r < D; ++r) pair(pk2(win[r][0], win[r][1]), nrx01, pk2(-ry[r], -ry[r]));
-                pair(pk2(win[0][2], win[1][2]), nrx22, pk2(-ry[0], -ry[1]));
-                const float z = win[2][2];
-                const float exs = fmaf(-z, rx[2], q.x), eys = fmaf(-z, ry[2], q.y), ezs = q.z - z;
-                nf += __saturatef(fmaf(-fmaf(exs, exs, fmaf(eys, eys, ezs * ezs)), 0x1p100f, r2b));
+                for (int r = 0; r < D; ++r)
+#pragma unroll
+                    for (int k = 0; k < W; ++k) pair(pk2(win[r][2 * k], win[r][2 * k + 1]), nrx2[k], pk2(-ry[r], -ry[r]));
+#pragma unroll
+                for (int k = 0; k < W; ++k) pair(pk2(win[2 * k][D - 1], win[2 * k + 1][D - 1]), nrxl, pk2(-ry[2 * k], -ry[2 * k + 1]));
+                one(D - 1, D - 1);
             } else {
 #pragma unroll
-                for (int r = 0; r < D; ++r) {
+                for (int r = 0; r < D; ++r)
 #pragma unroll
-                    for (int d = 0; d < D; ++d) {
-                        const float z = win[r][d];
-                        const float ex = fmaf(-z, rx[d], q.x), ey = fmaf(-z, ry[r], q.y), ez = q.z - z;
-                        nf += __saturatef(fmaf(-fmaf(ex, ex, fmaf(ey, ey, ez * ez)), 0x1p100f, r2b));
-                    }
-                }
+                    for (int e = 0; e < D; ++e) one(r, e);
             }
             n = (int)nf;
+        } else if (KIND == 1) {
+            // the same pairs; the terms are added row by row as pixel_ell adds them
+            const f32x2_t qx2 = pk2(q.x, q.x), qy2 = pk2(q.y, q.y), qz2 = pk2(q.z, q.z);
+            const f32x2_t nis2 = pk2(-L.inv2s2, -L.inv2s2);
+            auto add = [&](float z, float e) {
+                if (z >= 0.f) Ssum += e;
+            };
+            float last[2] = {0.f, 0.f};  // exponents of the last column's rows r, r + 1
+#pragma unroll
+            for (int r = 0; r < D; ++r) {
+#pragma unroll
+                for (int k = 0; k < W; ++k) {
+                    float ga, gb;
+                    upk2(mul2(dist2(pk2(win[r][2 * k], win[r][2 * k + 1]), nrx2[k], pk2(-ry[r], -ry[r]), qx2, qy2, qz2), nis2),
+                         ga, gb);
+                    add(win[r][2 * k], __expf(ga));
+                    add(win[r][2 * k + 1], __expf(gb));
+                }
+                if (r + 1 < D && r % 2 == 0) {
+                    upk2(mul2(dist2(pk2(win[r][D - 1], win[r + 1 < D ? r + 1 : r][D - 1]), nrxl, pk2(-ry[r], -ry[r + 1 < D ? r + 1 : r]), qx2,
+                                    qy2, qz2), nis2), last[0], last[1]);
+                } else if (r + 1 == D) {
+                    const float z = win[r][D - 1];
+                    const float ex = fmaf(-z, rx[D - 1], q.x), ey = fmaf(-z, ry[r], q.y), ez = q.z - z;
+                    last[0] = -fmaf(ex, ex, fmaf(ey, ey, ez * ez)) * L.inv2s2;
+                }
+                add(win[r][D - 1], __expf(last[r % 2]));
+            }
         } else {
 #pragma unroll
             for (int r = 0; r < D; ++r) {
@@ -201,12 +243,11 @@ __device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, 
                     const float z = win[r][d];
                     const float ex = fmaf(-z, rx[d], q.x), ey = fmaf(-z, ry[r], q.y), ez = q.z - z;
                     const float d2 = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-                    if (L.kind == 0) n += (z >= 0.f && d2 <= L.r2) ? 1 : 0;
-                    else if (z >= 0.f) Ssum += __expf(-d2 * L.inv2s2);
+                    n += (z >= 0.f && d2 <= L.r2) ? 1 : 0;
                 }
             }
         }
-        const float l = L.kind == 0 ? lut[n] : __logf(fmaf(L.bg, Ssum, L.a));
+        const float l = KIND == 0 ? lut[n] : __logf(fmaf(L.bg, Ssum, L.a));
         // a pixel without a point is skipped only now: a branch around the window loop costs
         // more than the loop (the lanes' pixels diverge)
         if (qe.x == 0.f) continue;
@@ -218,6 +259,15 @@ __device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, 
         }
     }
     return acc;
+}
+
+// score_column_kind of L.kind, for kernels that learn it as they run.
+template <int W, bool PAIRS = true>
+__device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
+                                              const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb,
+                                              unsigned long long *n_px, unsigned long long *n_pairs) {
+    return L.kind == 0 ? score_column_kind<W, 0, PAIRS>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, n_px, n_pairs)
+                       : score_column_kind<W, 1>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, n_px, n_pairs);
 }
 
 // z-buffer pixels per tile for a CTA of NT threads (measured: 3072 for 128 threads leaves room
@@ -681,7 +731,7 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
 // Scores the hypothesis whose pose thread 0 has put in sh.pose: returns, in thread 0, the
 // sum of l_i - l_i(bg) over the pixels whose window can see the object (0 when it is off
 // screen). All threads of the CTA must call it.
-template <bool STATS, int WT, int NT>
+template <bool STATS, int WT, int NT, int KIND>
 __device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, const float *s_lut, ScoreShared<NT> &sh,
                                             float4 *s_stage, unsigned *zb, float4 *lat, unsigned long long *cnt) {
     const Cam &c = S.cam;
@@ -700,9 +750,13 @@ __device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, co
                 const int seg = div_small(tid, tww), col = tid - seg * tww;
                 if (seg < nseg && col < tww) {
                     const int ya = qy0 + seg * rps, yb = min(ya + rps - 1, qy1);
-                    if (ya <= yb)
-                        acc += score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb,
-                                                STATS ? &cnt[6] : nullptr, STATS ? &cnt[7] : nullptr);
+                    unsigned long long *n_px = STATS ? &cnt[6] : nullptr, *n_pairs = STATS ? &cnt[7] : nullptr;
+                    if (ya <= yb) {
+                        if constexpr (KIND >= 0)
+                            acc += score_column_kind<WT, KIND>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, n_px, n_pairs);
+                        else
+                            acc += score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, n_px, n_pairs);
+                    }
                 }
             } else {
                 const int n_tile = tww * thh;
@@ -732,7 +786,9 @@ __device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, co
     return block_sum(acc, sh.red);
 }
 
-template <class PS, bool STATS, int WT, int NT, int MINB>
+// KIND: the likelihood's kind compiled in (-1: read from L, for the runtime half window): a
+// kernel that holds the loops of both is 1% slower for the 3x3 ball.
+template <class PS, bool STATS, int WT, int NT, int MINB, int KIND>
 __global__ void __launch_bounds__(NT, MINB)
     k_score(SceneView S, Lik L, PS P, int64_t n_hyp, float *out_ll) {
     constexpr int REG = score_region<NT>();
@@ -759,7 +815,7 @@ __global__ void __launch_bounds__(NT, MINB)
             if (STATS) ++cnt[0];
             pose12(P, h, sh.pose);
         }
-        const float tot = score_body<STATS, WT, NT>(S, L, s_lut, sh, s_stage, zb, lat, cnt);
+        const float tot = score_body<STATS, WT, NT, KIND>(S, L, s_lut, sh, s_stage, zb, lat, cnt);
         if (tid == 0) {
             out_ll[h] = (float)(*S.ll_bg + (double)tot);
             s_next = nxt;
@@ -821,7 +877,7 @@ __global__ void __launch_bounds__(NT, MINB)
                     if (s_item.pose_kind == 0) pose12(s_item.list, g - ib, sh.pose);
                     else pose12(s_item.grid, g - ib, sh.pose);
                 }
-                const float tot = score_body<false, WT, NT>(s_item.S, s_item.L, s_item.L.lut, sh, s_stage, zb, lat, nullptr);
+                const float tot = score_body<false, WT, NT, -1>(s_item.S, s_item.L, s_item.L.lut, sh, s_stage, zb, lat, nullptr);
                 if (tid == 0) s_item.out_ll[g - ib] = (float)(*s_item.S.ll_bg + (double)tot);
             }
         }
@@ -847,9 +903,15 @@ int launch_score_nt(const SceneView &sv, const Lik &L, PS P, int64_t n, float *l
     const int smem = score_region<NT>() * (int)sizeof(unsigned) + n_lat * (int)sizeof(float4);
     // work counting is compiled for one launch shape only (kStatsNT, kStatsMinB)
     constexpr bool ST = NT == kStatsNT && MINB == kStatsMinB;
-    auto kern = L.w == 1 ? k_score<PS, false, 1, NT, MINB> : (L.w == 2 ? k_score<PS, false, 2, NT, MINB> : k_score<PS, false, 0, NT, MINB>);
+    auto pick = [&](auto stats) {
+        constexpr bool B = decltype(stats)::value;
+        if (L.w == 1) return L.kind == 0 ? k_score<PS, B, 1, NT, MINB, 0> : k_score<PS, B, 1, NT, MINB, 1>;
+        if (L.w == 2) return L.kind == 0 ? k_score<PS, B, 2, NT, MINB, 0> : k_score<PS, B, 2, NT, MINB, 1>;
+        return k_score<PS, B, 0, NT, MINB, -1>;
+    };
+    auto kern = pick(std::false_type{});
     if constexpr (ST) {
-        if (sv.stats) kern = L.w == 1 ? k_score<PS, true, 1, NT, MINB> : (L.w == 2 ? k_score<PS, true, 2, NT, MINB> : k_score<PS, true, 0, NT, MINB>);
+        if (sv.stats) kern = pick(std::true_type{});
     }
     const int per_sm = kernel_ctas_per_sm(kern, NT, smem);
     // grid > 0: CTAs per SM requested by the tuning (capped by occupancy); 0: occupancy
