@@ -275,6 +275,10 @@ __global__ void __launch_bounds__(NT, MINB) k_render_fused(SceneView S, PoseList
 //       LL_h = LL_bg + sum_{i in box + w} (l_i - l_i(bg)).
 // MM = 1: miss mode 1 (pixels with id -1 carry no point). V = 4: step 1 reads 16-byte vectors
 // between the image's 16-byte boundaries (with MM the ids' too), else 1: pixel by pixel.
+// WHOLE: the images have no object slot (a moved camera's): they are scored in many tiles, and
+// the next tile's depths are copied to shared memory while one is scored (without ids to look
+// up on the way). The copies of one tile at a time were waited for in full (long scoreboard
+// 4.9 of 12 stall cycles): 2,048 images of 200x200, rendered and scored, 1,476 -> 1,446 us.
 __device__ __forceinline__ void box_note(int i, int W, int &x0, int &x1, int &y0, int &y1) {
     const int y = i / W, x = i - y * W;
     x0 = min(x0, x); x1 = max(x1, x); y0 = min(y0, y); y1 = max(y1, y);
@@ -366,12 +370,20 @@ __device__ __forceinline__ float score_column_ball3(const SceneView &S, const Li
     return acc;
 }
 
-template <int WT, int NT, int MINB, int V, int MM>
+__device__ __forceinline__ void async_copy4(float *dst, const float *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src));
+}
+__device__ __forceinline__ void async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+template <int WT, int NT, int MINB, int V, int MM, bool WHOLE>
 __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, const float *depth, const int *tid_in,
                                                           int64_t n_hyp, float *out_ll) {
     constexpr int REG = score_region<NT>();
     constexpr int U = 4;  // vector loads in flight per thread in the streaming pass
-    __shared__ __align__(16) float zd[REG];  // depths of the tile + w
+    constexpr bool PIPE = WHOLE && MM == 0;
+    __shared__ __align__(16) float zbuf[(PIPE ? 2 : 1) * REG];  // depths of the tile + w; PIPE: and of the next
     __shared__ float s_lut[kMaxLut];
     __shared__ float s_red[NT / 32];
     __shared__ int s_box[NT / 32][4];
@@ -478,47 +490,72 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
             const int sy0 = max(y0 - w, 0), sy1 = min(y1 + w, c.H - 1);
             const int tw = min(min(sx1 - sx0 + 1, min(S.tile_w, NT)), REG / (1 + 2 * w) - 2 * w);
             const int th = max(1, REG / (tw + 2 * w) - 2 * w);
+            // the depths of the tile at (tx0, ty0) + w into dst
+            auto stage = [&](int tx0, int ty0, float *dst) {
+                const int zx0 = max(tx0 - w, 0), zw = min(min(tx0 + tw - 1, sx1) + w, c.W - 1) - zx0 + 1;
+                const int zy0 = max(ty0 - w, 0), nz = zw * (min(min(ty0 + th - 1, sy1) + w, c.H - 1) - zy0 + 1);
+                const int dq = div_small(NT, zw), dr = NT - dq * zw;
+                int y = div_small(tid, zw), x = tid - y * zw;
+                for (int i = tid; i < nz; i += U * NT) {
+                    float d[U];
+#pragma unroll
+                    for (int u = 0; u < U; ++u) {
+                        d[u] = 0.f;
+                        if (i + u * NT < nz) {
+                            const int gi = (zy0 + y) * c.W + (zx0 + x);  // an image has at most 2^26 pixels
+                            if (PIPE) {
+                                async_copy4(dst + i + u * NT, img + gi);
+                            } else {
+                                d[u] = __ldg(img + gi);
+                                if (MM && __ldg(tim + gi) < 0) d[u] = -1.f;
+                            }
+                        }
+                        x += dr;
+                        y += dq;
+                        if (x >= zw) { x -= zw; ++y; }
+                    }
+                    if (!PIPE) {
+#pragma unroll
+                        for (int u = 0; u < U; ++u)
+                            if (i + u * NT < nz) dst[i + u * NT] = d[u];
+                    }
+                }
+                if (PIPE) async_commit();
+            };
+            if (PIPE) stage(sx0, sy0, zbuf);
+            int buf = 0;
             for (int ty0 = sy0; ty0 <= sy1; ty0 += th) {
                 for (int tx0 = sx0; tx0 <= sx1; tx0 += tw) {
                     const int tx1 = min(tx0 + tw - 1, sx1), ty1 = min(ty0 + th - 1, sy1);
-                    const int zx0 = max(tx0 - w, 0), zx1 = min(tx1 + w, c.W - 1);
-                    const int zy0 = max(ty0 - w, 0), zy1 = min(ty1 + w, c.H - 1);
-                    const int zw = zx1 - zx0 + 1, nz = zw * (zy1 - zy0 + 1);
-                    {
-                        const int dq = NT / zw, dr = NT - dq * zw;
-                        int y = tid / zw, x = tid - y * zw;
-                        for (int i = tid; i < nz; i += U * NT) {
-                            float d[U];
-#pragma unroll
-                            for (int u = 0; u < U; ++u) {
-                                d[u] = 0.f;
-                                if (i + u * NT < nz) {
-                                    const int gi = (zy0 + y) * c.W + (zx0 + x);  // an image has at most 2^26 pixels
-                                    d[u] = __ldg(img + gi);
-                                    if (MM && __ldg(tim + gi) < 0) d[u] = -1.f;
-                                }
-                                x += dr;
-                                y += dq;
-                                if (x >= zw) { x -= zw; ++y; }
-                            }
-#pragma unroll
-                            for (int u = 0; u < U; ++u)
-                                if (i + u * NT < nz) zd[i + u * NT] = d[u];
+                    const int zx0 = max(tx0 - w, 0), zx1 = min(tx1 + w, c.W - 1), zy0 = max(ty0 - w, 0);
+                    const int zw = zx1 - zx0 + 1;
+                    const float *zd = zbuf + buf * REG;
+                    if (PIPE) {
+                        const bool wrap = tx0 + tw > sx1;
+                        const int nx = wrap ? sx0 : tx0 + tw, ny = wrap ? ty0 + th : ty0;
+                        buf ^= 1;
+                        if (ny <= sy1) {
+                            stage(nx, ny, zbuf + buf * REG);
+                            async_wait<1>();
+                        } else {
+                            async_wait<0>();
                         }
+                    } else {
+                        stage(tx0, ty0, zbuf);
                     }
                     __syncthreads();
                     const int tww = tx1 - tx0 + 1, thh = ty1 - ty0 + 1;
                     if (WT > 0) {
                         // thread -> (column, run of rows)
-                        const int nseg = max(1, NT / tww);
-                        const int rps = (thh + nseg - 1) / nseg;
-                        const int seg = tid / tww, col = tid - seg * tww;
+                        const int nseg = max(1, div_small(NT, tww));
+                        const int rps = div_small(thh + nseg - 1, nseg);
+                        const int seg = div_small(tid, tww), col = tid - seg * tww;
                         if (seg < nseg && col < tww) {
                             const int ya = ty0 + seg * rps, yb = min(ya + rps - 1, ty1);
                             if (ya <= yb)
                                 acc += WT == 1 && ball3
                                            ? score_column_ball3(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb)
-                                           : score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, nullptr,
+                                           : score_column<WT, !WHOLE>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, nullptr,
                                                               nullptr);
                         }
                     } else {
@@ -617,8 +654,8 @@ static void launch_score_fused(const SceneView &sv, const Lik &L, const float *d
                                float *ll, int grid, cudaStream_t s) {
     const bool mm = L.miss_mode == 1;
     constexpr int MB = score_fused_minb<WT>(WHOLE);
-    auto kern = !mm ? k_score_fused<WT, kMatNT, MB, 4, 0>
-                    : (same_offset16(depth, tid) ? k_score_fused<WT, kMatNT, MB, 4, 1> : k_score_fused<WT, kMatNT, MB, 1, 1>);
+    auto kern = !mm ? k_score_fused<WT, kMatNT, MB, 4, 0, WHOLE>
+                    : (same_offset16(depth, tid) ? k_score_fused<WT, kMatNT, MB, 4, 1, WHOLE> : k_score_fused<WT, kMatNT, MB, 1, 1, WHOLE>);
     if (sv.work) cudaMemsetAsync(sv.work, 0, sizeof(unsigned long long), s);
     kern<<<persistent_grid(kern, kMatNT, 0, n, grid), kMatNT, 0, s>>>(sv, L, depth, tid, n, ll);
 }
@@ -629,6 +666,7 @@ int launch_score_depth(const SceneView &sv, const Lik &L, const float *depth, co
     const bool whole = sv.mesh.n_full <= 0;  // no object slot
     if (L.w == 1 && whole) launch_score_fused<1, true>(sv, L, depth, tid, n, ll, grid, s);
     else if (L.w == 1) launch_score_fused<1, false>(sv, L, depth, tid, n, ll, grid, s);
+    else if (L.w == 2 && whole) launch_score_fused<2, true>(sv, L, depth, tid, n, ll, grid, s);
     else if (L.w == 2) launch_score_fused<2, false>(sv, L, depth, tid, n, ll, grid, s);
     else launch_score_fused<0, false>(sv, L, depth, tid, n, ll, grid, s);
     return 1;
