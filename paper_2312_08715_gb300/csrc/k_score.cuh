@@ -251,7 +251,9 @@ __device__ __forceinline__ float score_column_kind(const SceneView &S, const Lik
         // a pixel without a point is skipped only now: a branch around the window loop costs
         // more than the loop (the lanes' pixels diverge)
         if (qe.x == 0.f) continue;
-        acc += l - qe.y;
+        // rounded as it stands: the compiler may not fold the logarithm's last product into the
+        // difference, which is 0 for a term equal to the background's
+        acc += __fsub_rn(l, qe.y);
         if (n_px) {
             ++*n_px;
             *n_pairs += (unsigned long long)((min(y + W, c.H - 1) - max(y - W, 0) + 1) *
