@@ -431,15 +431,19 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
 // Launch shape of a score launch (the code of launch_score and the tile width) when none was
 // set or tuned: single calls, each stage of an enumeration and batched launches. Shapes differ
 // in the order of the FP32 sums (1e-8 of a score); a server, whose results must not depend on
-// what shares a batch, fixes one. The CTA size follows the work of a hypothesis, estimated in microseconds of an
-// SM from the slot object's rectangles q and its size D in pixels at the scene's pose:
+// what shares a batch, fixes one. The CTA size follows the work of a hypothesis, estimated in
+// microseconds of an SM from the slot object's rectangles q and its size D in pixels at the scene's pose:
 //   c = 0.35 + 0.00113 q + D^2 (0.0003 + e (2w+1)^2), e = 0.00006 (ball) or 0.0001 (Gaussian),
 // a fit to a sweep of 33 shapes over 64x48 to 320x240 images, objects of 600 to 12,000 cells
 // and both likelihoods. Up to 1.3 us a hypothesis 32 threads are the fastest (30,000
 // hypotheses of 873 cells at 160x120: 175 us; 64: 205, 128: 236, 256: 398), up to 2.6 64
-// (5,109 cells, 160x120: 453; 128: 463, 256: 696), up to 5.8 128 (17,536 cells,
-// 160x120: 865; 64: 971, 256: 1,094), above 256 with tiles of 128 pixels (320x240: 1,867;
-// 256 threads with 64-pixel tiles 2,337, 128 threads 2,367). A call of few hypotheses takes
+// (5,109 cells, 160x120: 453; 128: 463, 256: 696), above 128, or 256 with tiles of 128 pixels
+// where the footprint does not fit the 3,072-pixel z-buffer of 128 threads and would be drawn
+// tile by tile. For one object that line lies at D + 2w = 63, whatever the likelihood (112
+// points of 64x48 to 320x240 images, objects of 800 to 15,000 cells; 3,000 hypotheses, us at
+// 128 and 256 threads: D = 59.5, w = 1 103 and 107; 62.8 119 and 108; 72 165 and 134; 58.6,
+// w = 2 127 and 145; 59.5 147 and 142; a line by c had cost 5x5 windows up to 18%); a batch of
+// scenes, whose sizes differ, takes 256 above c = 5.8. A call of few hypotheses takes
 // larger CTAs, so that each SM still has some 600 threads: 1,000 hypotheses of the first
 // object take 15 us with 128 threads, 24 with 256; 300 take 12 with 256, 13 with 64.
 // Calls that kept 256 threads and 64-pixel tiles before: 1,000 hypotheses at 64x48 36 -> 26 us,
@@ -449,19 +453,22 @@ struct ScoreShape {
     int code, tile_w;
 };
 
-double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L) {
+// c, and in *side_px D + 2w
+double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L, double *side_px = nullptr) {
     const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
     double d2 = 0;
     for (int k = 0; k < 3; ++k) d2 += (double)(m.hi[k] - m.lo[k]) * (m.hi[k] - m.lo[k]);
     const double z = std::max((double)ctx->obj_z[slot], 0.5 * std::sqrt(d2) + ctx->cam.near_z);
     const double f = std::max(ctx->cam.fx, ctx->cam.fy), side = 2.0 * L.w + 1.0;
     const double px2 = std::min(d2 * f * f / (z * z), (double)ctx->cam.W * ctx->cam.H);
+    if (side_px) *side_px = std::sqrt(px2) + 2.0 * L.w;
     return 0.35 + 0.00113 * m.n_quads + px2 * (0.0003 + (L.kind == 0 ? 0.00006 : 0.0001) * side * side);
 }
 
-ScoreShape shape_of_cost(double cost, int64_t n) {
+// large: the footprints do not fit the z-buffer of 128 threads
+ScoreShape shape_of_cost(double cost, bool large, int64_t n) {
     const int64_t want = 152 * 600;  // threads that keep the device busy
-    int nt = cost <= 1.3 ? 32 : (cost <= 2.6 ? 64 : (cost <= 5.8 ? 128 : 256));
+    int nt = cost <= 1.3 ? 32 : (cost <= 2.6 ? 64 : (large ? 256 : 128));
     while (nt < 256 && n * nt < want) nt *= 2;
     const int code = nt == 128 ? 1 : (nt == 64 ? 2 : (nt == 32 ? 3 : 0));
     return ScoreShape{code << 8, nt == 256 ? 128 : (nt == 128 ? 96 : nt)};
@@ -471,7 +478,9 @@ ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, int64_t n)
     const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
     // half windows without a compiled-in scorer and triangle meshes keep the general shape
     if (ctx->shape_set || m.n_quads <= 0 || L.w < 1 || L.w > 2) return ScoreShape{ctx->score_code(), ctx->tile_w};
-    return shape_of_cost(score_cost(ctx, slot, L), n);
+    double side = 0;
+    const double cost = score_cost(ctx, slot, L, &side);
+    return shape_of_cost(cost, side > 63.0, n);
 }
 
 // The shape of one batched launch: of the cost of a hypothesis, weighted by the time its scene
@@ -490,7 +499,7 @@ ScoreShape pick_shape_multi(const b3d_ctx *owner, int n_items, Scene scene, Slot
         tc += c * c * (double)hyps(i);
         total += hyps(i);
     }
-    return t > 0 ? shape_of_cost(tc / t, total) : set;
+    return t > 0 ? shape_of_cost(tc / t, tc / t > 5.8, total) : set;
 }
 
 // A hypothesis counter for one persistent launch (its launcher zeroes it): a ring, so launches
