@@ -408,7 +408,8 @@ b3d_status b3d_autotune(b3d_ctx *ctx, int32_t obj_slot, const float *centre_pose
 
 /* Autotuner for the batched form: times b3d_enumerate_multi on these items (owner, items and
  * lik as there) for the owner's current launch shape and for 128- or 256-thread CTAs with 64-
- * or 128-pixel tiles, then the fastest shape with 1 to 32 hypotheses per work-queue grab;
+ * or 128-pixel tiles (an owner that was not tuned: also for the smaller shapes its launches
+ * choose among), then the fastest shape with 1 to 32 hypotheses per work-queue grab;
  * keeps the fastest tuning in the owner and returns it in *best (may be NULL). The items'
  * outputs hold the last timed run's results. Synchronises the stream (not for use while
  * capturing a graph). No counterpart in the paper: the launch shape is a property of this

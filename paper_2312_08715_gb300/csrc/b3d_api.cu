@@ -465,13 +465,15 @@ double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L, double *side_p
     return 0.35 + 0.00113 * m.n_quads + px2 * (0.0003 + (L.kind == 0 ? 0.00006 : 0.0001) * side * side);
 }
 
+int auto_tile_w(int cta_threads) { return cta_threads == 256 ? 128 : (cta_threads == 128 ? 96 : cta_threads); }
+
 // large: the footprints do not fit the z-buffer of 128 threads
 ScoreShape shape_of_cost(double cost, bool large, int64_t n) {
     const int64_t want = 152 * 600;  // threads that keep the device busy
     int nt = cost <= 1.3 ? 32 : (cost <= 2.6 ? 64 : (large ? 256 : 128));
     while (nt < 256 && n * nt < want) nt *= 2;
     const int code = nt == 128 ? 1 : (nt == 64 ? 2 : (nt == 32 ? 3 : 0));
-    return ScoreShape{code << 8, nt == 256 ? 128 : (nt == 128 ? 96 : nt)};
+    return ScoreShape{code << 8, auto_tile_w(nt)};
 }
 
 ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, int64_t n) {
@@ -2036,9 +2038,11 @@ b3d_status b3d_autotune_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_ite
         owner->tile_w = t.tile_w; owner->cta_threads = t.cta_threads; owner->ctas_per_sm = t.ctas_per_sm;
         owner->high_occupancy = t.high_occupancy; owner->batch_chunk = t.batch_chunk;
     };
+    const bool was_set = owner->shape_set;
     // one untimed pass with the current tuning: sizes the scratch and builds every item's tables
     b3d_status st = b3d_enumerate_multi(owner, n_items, items, lik, stream);
     if (st != B3D_OK) return st;
+    owner->shape_set = true;  // the candidates' shapes, not pick_shape_multi's
     cudaEvent_t e0 = take_event(owner), e1 = take_event(owner);
     auto timed = [&](const b3d_tuning &t, float *ms) -> b3d_status {
         apply(t);
@@ -2054,10 +2058,13 @@ b3d_status b3d_autotune_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_ite
         cudaEventElapsedTime(ms, e0, e1);
         return B3D_OK;
     };
-    // launch shapes: the current one and 128- or 256-thread CTAs with 64- or 128-pixel tiles
+    // launch shapes: the current one and 128- or 256-thread CTAs with 64- or 128-pixel tiles;
+    // of an owner that was not tuned also the others that its launches may have been taking
     std::vector<b3d_tuning> shapes{saved};
     for (int nt : {128, 256})
         for (int tw : {64, 128}) shapes.push_back(b3d_tuning{tw, nt, 0, 0, saved.batch_chunk});
+    if (!was_set)
+        for (int nt : {32, 64, 128}) shapes.push_back(b3d_tuning{auto_tile_w(nt), nt, 0, 0, saved.batch_chunk});
     b3d_tuning win = saved;
     float win_ms = INFINITY;
     for (const b3d_tuning &t : shapes) {
@@ -2078,10 +2085,10 @@ b3d_status b3d_autotune_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_ite
     owner->event_pool.push_back(e1);
     if (st != B3D_OK) {
         apply(saved);
+        owner->shape_set = was_set;
         return st;
     }
     apply(win);
-    owner->shape_set = true;
     if (best) *best = win;
     return B3D_OK;
 }
