@@ -270,9 +270,9 @@ b3d_status b3d_enumerate_c2f(b3d_ctx *ctx, int32_t obj_slot, const float *centre
  * persistent launch whose CTAs take batch_chunk hypotheses at a time from a work queue over
  * (scene, hypothesis chunk). Items may differ in image size, meshes, object slot and
  * hypothesis count; the likelihood is shared (its frustum volume is each scene's own).
- * Scores equal those of b3d_score_batch on each scene alone (bit for bit under the same
- * b3d_set_tuning; a context that was not tuned picks its launch shape by the size of the work,
- * and shapes differ in FP32 summation order). The owner's context supplies
+ * Scores equal those of b3d_score_batch on each scene alone, bit for bit: with half windows 1
+ * and 2 whatever the tunings (a score does not depend on the launch shape), with others under
+ * the same tuning (the FP32 sum follows the shape). The owner's context supplies
  * the launch shape (b3d_tuning) and the scratch; scratch is sized on first use, after
  * which the call can be captured into a CUDA graph (it allocates nothing and only copies its
  * descriptors from pinned host memory). */
@@ -290,7 +290,7 @@ b3d_status b3d_score_multi(b3d_ctx *owner, int32_t n_items, const b3d_score_item
 /* Batched coarse-to-fine enumeration: every item runs b3d_enumerate_c2f on its own scene and
  * schedule (all schedules with the same number of stages); each stage is one batched score
  * launch, one batched log-sum-exp + resampling launch and one batched selection launch over
- * all items. Outputs per item as b3d_enumerate_c2f. An item's centre may be read from
+ * all items. Outputs per item as b3d_enumerate_c2f, the same bits as far as b3d_score_multi's. An item's centre may be read from
  * device memory (centre_dev, copied before the first stage, so it may point into the
  * item's own particles_dev). Same graph-capture rule as b3d_score_multi. */
 typedef struct {
@@ -386,7 +386,8 @@ b3d_status b3d_score_noise_batch(b3d_ctx *ctx, int32_t obj_slot, int64_t n_hyp, 
  * that more CTAs fit on an SM, 0 the regular one; batch_chunk (1..1024): see b3d_score_multi.
  * Until b3d_set_tuning or an autotuner is called on a context, its score launches with half
  * windows 1 and 2 of voxel meshes take a CTA size and tile width chosen by the size of the
- * object, the image and the batch; b3d_get_tuning then reports the general default. */
+ * object, the image and the batch (which changes their time, not their scores); b3d_get_tuning
+ * then reports the general default. Setting any field sets the shape, for the context's life. */
 typedef struct {
     int32_t tile_w;
     int32_t cta_threads;

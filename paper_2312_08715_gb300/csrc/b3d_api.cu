@@ -429,9 +429,8 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
 }
 
 // Launch shape of a score launch (the code of launch_score and the tile width) when none was
-// set or tuned: single calls, each stage of an enumeration and batched launches. Shapes differ
-// in the order of the FP32 sums (1e-8 of a score); a server, whose results must not depend on
-// what shares a batch, fixes one. The CTA size follows the work of a hypothesis, estimated in
+// set or tuned: single calls, each stage of an enumeration and batched launches, with half windows
+// whose scores do not depend on the shape (FixedSum in k_score.cuh). The CTA size follows the work of a hypothesis, estimated in
 // microseconds of an SM from the slot object's rectangles q and its size D in pixels at the scene's pose:
 //   c = 0.35 + 0.00113 q + D^2 (0.0003 + e (2w+1)^2), e = 0.00006 (ball) or 0.0001 (Gaussian),
 // a fit to a sweep of 33 shapes over 64x48 to 320x240 images, objects of 600 to 12,000 cells
@@ -478,7 +477,8 @@ ScoreShape shape_of_cost(double cost, bool large, int64_t n) {
 
 ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, int64_t n) {
     const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
-    // half windows without a compiled-in scorer and triangle meshes keep the general shape
+    // half windows without a compiled-in scorer (an FP32 sum in the shape's order) and triangle
+    // meshes keep the general shape
     if (ctx->shape_set || m.n_quads <= 0 || L.w < 1 || L.w > 2) return ScoreShape{ctx->score_code(), ctx->tile_w};
     double side = 0;
     const double cost = score_cost(ctx, slot, L, &side);

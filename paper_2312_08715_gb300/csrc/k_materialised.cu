@@ -552,11 +552,12 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                         const int seg = div_small(tid, tww), col = tid - seg * tww;
                         if (seg < nseg && col < tww) {
                             const int ya = ty0 + seg * rps, yb = min(ya + rps - 1, ty1);
-                            if (ya <= yb)
-                                acc += WT == 1 && ball3
-                                           ? score_column_ball3(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb)
-                                           : score_column<WT, !WHOLE>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, nullptr,
-                                                              nullptr);
+                            if (ya <= yb) {
+                                FloatSum sum;
+                                if (WT == 1 && ball3) sum.v = score_column_ball3(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb);
+                                else score_column<WT, !WHOLE>(S, L, s_lut, c, zd, zx0, zy0, zw, tx0 + col, ya, yb, sum, nullptr, nullptr);
+                                acc += sum.v;
+                            }
                         }
                     } else {
                         const int n_t = tww * thh;

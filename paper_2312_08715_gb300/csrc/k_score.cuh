@@ -50,7 +50,7 @@ inline int score_sm_count() {
 //  3. per screen tile: start a 32-bit z-buffer of depth bits from the fixed objects' depths,
 //     rasterise into it with atomicMin (the score depends only on the nearest depth, so no
 //     triangle id rides along), score the tile's observed pixels against their background terms.
-//  4. block reduction to one log-likelihood.
+//  4. block reduction to one log-likelihood (FixedSum: the same bits under every launch shape).
 // STATS: count the work done (hypotheses, projected vertices/corners, primitives, pixel
 // tests, fragments, composited pixels, scored pixels, window pairs) into S.stats.
 // WT: the half window compiled in (1 or 2: sliding-window scoring), 0: runtime L.w.
@@ -114,18 +114,52 @@ __device__ __forceinline__ f32x2_t dist2(f32x2_t z, f32x2_t nrx, f32x2_t nry, f3
     return fma2(ex, ex, fma2(ey, ey, mul2(ez, ez)));
 }
 
-// Sum of l_i - l_i(bg) over pixel column x, rows [ya, yb], with the (2W+1)^2 window of
-// rendered depths slid down the column in registers. Window slots outside the image (and
+// Where a column's differences l_i - l_i(bg) go. FloatSum: a float.
+struct FloatSum {
+    float v = 0.f;
+    __device__ __forceinline__ void add(float d, bool) { v += d; }
+};
+
+// The differences of one tile's pixels as multiples of 2^-28 in integers, so that their sum over
+// threads and tiles has one value however the pixels were shared out: a score has the same bits
+// under every launch shape, and with it in a batch, in a part of a list and in a server. The high
+// part counts 2^-9, the low part what is left, both read off the mantissa of a sum with a
+// constant; the error is 2^-29 at most, and none for a difference of 2^-5 and more (in float the
+// partial sums of some hundred were rounded to 2^-17). A ball's terms are logarithms that the host
+// formed, at most some 780 apart; a Gaussian's can be infinite or NaN under extreme parameters and
+// then goes into `wild`, a plain float. A thread has at most 128 rows of a tile, a warp 4,096
+// differences, so the 32-bit sums of a warp stay below 2^31. Against a float sum (GB300, us):
+// 145,800 hypotheses at 160x120 2,068 -> 2,094, 31,250 at 320x240 1,095 -> 1,115, Gaussian 5x5 the same.
+struct FixedSum {
+    float *wild;  // in shared memory
+    int hi = 0, lo = 0;
+    __device__ __forceinline__ void add(float d, bool can_be_wild) {
+        constexpr float kHi = 0x1.8p14f, kLo = 0x1.8p-5f;  // their last places: 2^-9 and 2^-28
+        if (can_be_wild && !(fabsf(d) < 512.f)) {
+            atomicAdd(wild, d);
+            d = 0.f;
+        }
+        const float s = __fadd_rn(d, kHi);
+        hi += __float_as_int(s) - __float_as_int(kHi);
+        // d - (s - kHi) + kLo: the difference from s and the two constants are exact, the sum with d rounds
+        lo += __float_as_int(__fadd_rn(d, __fsub_rn(kHi + kLo, s))) - __float_as_int(kLo);
+    }
+};
+constexpr int kFixedShift = 19;  // hi counts 2^19 of lo's units
+constexpr double kFixedUnit = 0x1p-28;
+
+// Adds d = l_i - l_i(bg) over pixel column x, rows [ya, yb], to `sum`, with the (2W+1)^2 window
+// of rendered depths slid down the column in registers. Window slots outside the image (and
 // pixels without a point) hold -1 and contribute nothing; the terms are formed in the same
 // order and by the same expressions as pixel_ell, so unchanged pixels give 0 exactly.
 // KIND: L.kind compiled in. The window's elements are taken in packed pairs, Gaussian or ball
 // (PAIRS = false: the 5x5 ball one by one): issue-bound, so a pair saves 7 of its 14 FP32
 // instructions (GB300, us: 20,000 hypotheses at 160x120, Gaussian 5x5 874 -> 765, 3x3 468 ->
 // 440; ball 5x5 563 -> 552; 16,001 Gaussian 5x5 at 150x113 377 -> 333).
-template <int W, int KIND, bool PAIRS = true>
-__device__ __forceinline__ float score_column_kind(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
-                                              const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb,
-                                              unsigned long long *n_px, unsigned long long *n_pairs) {
+template <int W, int KIND, bool PAIRS = true, class Sum>
+__device__ __forceinline__ void score_column_kind(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
+                                                  const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb, Sum &sum,
+                                                  unsigned long long *n_px, unsigned long long *n_pairs) {
     constexpr int D = 2 * W + 1;
     float rx[D], ry[D], win[D][D];
     bool colok[D];
@@ -145,7 +179,6 @@ __device__ __forceinline__ float score_column_kind(const SceneView &S, const Lik
         load_row(ya - W + r - 1, win[r]);
         ry[r] = ((float)(ya - W + r - 1) + 0.5f - c.cy) * c.inv_fy;
     }
-    float acc = 0.f;
     const bool ball_skips_empty = L.r2 < 0.25f;
     const float r2b = __int_as_float(__float_as_int(L.r2) + 1) * 0x1p100f;  // (next float above r2) 2^100
     const float rxc = rx[W];  // the column's own ray
@@ -253,23 +286,22 @@ __device__ __forceinline__ float score_column_kind(const SceneView &S, const Lik
         if (qe.x == 0.f) continue;
         // rounded as it stands: the compiler may not fold the logarithm's last product into the
         // difference, which is 0 for a term equal to the background's
-        acc += __fsub_rn(l, qe.y);
+        sum.add(__fsub_rn(l, qe.y), KIND == 1);
         if (n_px) {
             ++*n_px;
             *n_pairs += (unsigned long long)((min(y + W, c.H - 1) - max(y - W, 0) + 1) *
                                              (min(x + W, c.W - 1) - max(x - W, 0) + 1));
         }
     }
-    return acc;
 }
 
 // score_column_kind of L.kind, for kernels that learn it as they run.
-template <int W, bool PAIRS = true>
-__device__ __forceinline__ float score_column(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
-                                              const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb,
-                                              unsigned long long *n_px, unsigned long long *n_pairs) {
-    return L.kind == 0 ? score_column_kind<W, 0, PAIRS>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, n_px, n_pairs)
-                       : score_column_kind<W, 1>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, n_px, n_pairs);
+template <int W, bool PAIRS = true, class Sum>
+__device__ __forceinline__ void score_column(const SceneView &S, const Lik &L, const float *lut, const Cam &c,
+                                             const float *zd, int zx0, int zy0, int zw, int x, int ya, int yb, Sum &sum,
+                                             unsigned long long *n_px, unsigned long long *n_pairs) {
+    if (L.kind == 0) score_column_kind<W, 0, PAIRS>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, sum, n_px, n_pairs);
+    else score_column_kind<W, 1>(S, L, lut, c, zd, zx0, zy0, zw, x, ya, yb, sum, n_px, n_pairs);
 }
 
 // z-buffer pixels per tile for a CTA of NT threads (measured: 3072 for 128 threads leaves room
@@ -316,6 +348,8 @@ struct ScoreShared {
     int flags;    // bit 0: on screen, bit 1: rectangle path, bit 2: whole object beyond near
     int rng[13];  // class first rectangles [6], exclusive prefix of counts [6], total
     float red[NT / 32];
+    unsigned fix[2];  // low and high word of the hypothesis's FixedSum,
+    float wild;       // and its terms outside
     int own[NT];  // per warp: the lane whose candidate run starts at each position of a window
 };
 
@@ -732,15 +766,24 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
 
 // Scores the hypothesis whose pose thread 0 has put in sh.pose: returns, in thread 0, the
 // sum of l_i - l_i(bg) over the pixels whose window can see the object (0 when it is off
-// screen). All threads of the CTA must call it.
+// screen). All threads of the CTA must call it. With a half window compiled in the sum is a
+// FixedSum: each warp's first lane adds its part of a tile to the 64 bits of sh.fix (two 32-bit
+// additions, the carry from the old low word), and the barrier that ends a tile orders them before
+// thread 0 reads. (A slot of sh.fix per warp took the 3x3 ball from 72 to 75 registers, 7 to 6 CTAs
+// per SM: 7%.)
 template <bool STATS, int WT, int NT, int KIND>
-__device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, const float *s_lut, ScoreShared<NT> &sh,
+__device__ __forceinline__ double score_body(const SceneView &S, const Lik &L, const float *s_lut, ScoreShared<NT> &sh,
                                             float4 *s_stage, unsigned *zb, float4 *lat, unsigned long long *cnt) {
     const Cam &c = S.cam;
     constexpr int nt = NT;
-    const int tid = threadIdx.x;
+    const int tid = threadIdx.x, lane = tid & 31;
     const int w = WT > 0 ? WT : L.w;
+    const bool can_be_wild = KIND == 1 || (KIND < 0 && L.kind == 1);
     float acc = 0.f;
+    if (WT > 0 && tid == 0) {  // ordered by render_tiles' first barrier
+        sh.fix[0] = sh.fix[1] = 0;
+        sh.wild = 0.f;
+    }
     const bool drawn = render_tiles<STATS, NT>(
         S, w, L.miss_mode, sh, s_stage, zb, lat, cnt,
         [&](const float *zd, int zx0, int zy0, int zw, int qx0, int qx1, int qy0, int qy1, int, int, int, int) {
@@ -750,15 +793,22 @@ __device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, co
                 const int nseg = max(1, div_small(NT, tww));
                 const int rps = div_small(thh + nseg - 1, nseg);
                 const int seg = div_small(tid, tww), col = tid - seg * tww;
+                FixedSum sum{&sh.wild};
                 if (seg < nseg && col < tww) {
                     const int ya = qy0 + seg * rps, yb = min(ya + rps - 1, qy1);
                     unsigned long long *n_px = STATS ? &cnt[6] : nullptr, *n_pairs = STATS ? &cnt[7] : nullptr;
                     if (ya <= yb) {
                         if constexpr (KIND >= 0)
-                            acc += score_column_kind<WT, KIND>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, n_px, n_pairs);
+                            score_column_kind<WT, KIND>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, sum, n_px, n_pairs);
                         else
-                            acc += score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, n_px, n_pairs);
+                            score_column<WT>(S, L, s_lut, c, zd, zx0, zy0, zw, qx0 + col, ya, yb, sum, n_px, n_pairs);
                     }
+                }
+                const int hi = __reduce_add_sync(0xffffffffu, sum.hi), lo = __reduce_add_sync(0xffffffffu, sum.lo);
+                if (lane == 0) {
+                    const long long v = ((long long)hi << kFixedShift) + lo;
+                    const unsigned low = (unsigned)v, old = atomicAdd(&sh.fix[0], low);
+                    atomicAdd(&sh.fix[1], (unsigned)(v >> 32) + (old + low < low ? 1u : 0u));
                 }
             } else {
                 const int n_tile = tww * thh;
@@ -784,8 +834,16 @@ __device__ __forceinline__ float score_body(const SceneView &S, const Lik &L, co
                 }
             }
         });
-    if (!drawn) return 0.f;
-    return block_sum(acc, sh.red);
+    if (!drawn) return 0.0;
+    if (WT > 0) {
+        double tot = 0.0;
+        if (tid == 0) {
+            tot = (double)(long long)(((unsigned long long)sh.fix[1] << 32) | sh.fix[0]) * kFixedUnit;
+            if (can_be_wild) tot += (double)sh.wild;
+        }
+        return tot;
+    }
+    return (double)block_sum(acc, sh.red);
 }
 
 // KIND: the likelihood's kind compiled in (-1: read from L, for the runtime half window): a
@@ -817,9 +875,9 @@ __global__ void __launch_bounds__(NT, MINB)
             if (STATS) ++cnt[0];
             pose12(P, h, sh.pose);
         }
-        const float tot = score_body<STATS, WT, NT, KIND>(S, L, s_lut, sh, s_stage, zb, lat, cnt);
+        const double tot = score_body<STATS, WT, NT, KIND>(S, L, s_lut, sh, s_stage, zb, lat, cnt);
         if (tid == 0) {
-            out_ll[h] = (float)(*S.ll_bg + (double)tot);
+            out_ll[h] = (float)(*S.ll_bg + tot);
             s_next = nxt;
         }
         __syncthreads();  // the next write of s_next comes after score_body's barriers
@@ -879,8 +937,8 @@ __global__ void __launch_bounds__(NT, MINB)
                     if (s_item.pose_kind == 0) pose12(s_item.list, g - ib, sh.pose);
                     else pose12(s_item.grid, g - ib, sh.pose);
                 }
-                const float tot = score_body<false, WT, NT, -1>(s_item.S, s_item.L, s_item.L.lut, sh, s_stage, zb, lat, nullptr);
-                if (tid == 0) s_item.out_ll[g - ib] = (float)(*s_item.S.ll_bg + (double)tot);
+                const double tot = score_body<false, WT, NT, -1>(s_item.S, s_item.L, s_item.L.lut, sh, s_stage, zb, lat, nullptr);
+                if (tid == 0) s_item.out_ll[g - ib] = (float)(*s_item.S.ll_bg + tot);
             }
         }
     }
