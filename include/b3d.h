@@ -386,8 +386,10 @@ b3d_status b3d_score_noise_batch(b3d_ctx *ctx, int32_t obj_slot, int64_t n_hyp, 
  * that more CTAs fit on an SM, 0 the regular one; batch_chunk (1..1024): see b3d_score_multi.
  * Until b3d_set_tuning or an autotuner is called on a context, its score launches with half
  * windows 1 and 2 of voxel meshes take a CTA size and tile width chosen by the size of the
- * object, the image and the batch (which changes their time, not their scores); b3d_get_tuning
- * then reports the general default. Setting any field sets the shape, for the context's life. */
+ * object at its centre or scene pose, the image and the batch (which changes their time, not
+ * their scores), or the general default where the host has no such pose (after
+ * b3d_set_object_pose_dev, or one that is not before the camera); b3d_get_tuning then reports the
+ * general default. Setting any field sets the shape, for the context's life. */
 typedef struct {
     int32_t tile_w;
     int32_t cta_threads;

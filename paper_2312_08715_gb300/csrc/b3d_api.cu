@@ -122,7 +122,7 @@ struct b3d_ctx {
     float *d_centre = nullptr;  // [3][16]: two ping-pong centres and one expand scratch
     std::map<std::tuple<int, int, float>, float *> rot_cache;
 
-    std::vector<float> obj_z;  // camera depth of each object at b3d_set_scene (see pick_shape)
+    std::vector<float> obj_z;  // camera depth of each object at b3d_set_scene, NaN once its pose came from the device (see pick_shape)
 
     // launch shape of the score kernel; until it is set or tuned, launches take pick_shape's
     bool shape_set = false;
@@ -430,8 +430,10 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
 
 // Launch shape of a score launch (the code of launch_score and the tile width) when none was
 // set or tuned: single calls, each stage of an enumeration and batched launches, with half windows
-// whose scores do not depend on the shape (FixedSum in k_score.cuh). The CTA size follows the work of a hypothesis, estimated in
-// microseconds of an SM from the slot object's rectangles q and its size D in pixels at the scene's pose:
+// whose scores do not depend on the shape (FixedSum in k_score.cuh). The CTA size follows the
+// work of a hypothesis, estimated in microseconds of an SM from the slot object's rectangles q and
+// its size D in pixels at the depth of the grid's centre where the host knows it, else of the
+// scene's pose:
 //   c = 0.35 + 0.00113 q + D^2 (0.0003 + e (2w+1)^2), e = 0.00006 (ball) or 0.0001 (Gaussian),
 // a fit to a sweep of 33 shapes over 64x48 to 320x240 images, objects of 600 to 12,000 cells
 // and both likelihoods. Up to 1.3 us a hypothesis 32 threads are the fastest (30,000
@@ -444,7 +446,11 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
 // w = 2 127 and 145; 59.5 147 and 142; a line by c had cost 5x5 windows up to 18%); a batch of
 // scenes, whose sizes differ, takes 256 above c = 5.8. A call of few hypotheses takes
 // larger CTAs, so that each SM still has some 600 threads: 1,000 hypotheses of the first
-// object take 15 us with 128 threads, 24 with 256; 300 take 12 with 256, 13 with 64.
+// object take 15 us with 128 threads, 24 with 256; 300 take 12 with 256, 13 with 64. Where the
+// depth is not known (an object whose pose came from the device, or whose scene pose does not lie
+// before the camera: a placeholder) the general shape stays: a depth 16 times too large made a
+// search of 3,750 hypotheses of 600 cells 404 us long, the general shape takes 319 and the right
+// depth's 291.
 // Calls that kept 256 threads and 64-pixel tiles before: 1,000 hypotheses at 64x48 36 -> 26 us,
 // 16,001 smooth 5x5 ones at 150x113 470 -> 367, 31,250 at 320x240 1,569 -> 1,324, eight scenes
 // batched 721 -> 595, a tracking step at 320x240 370 -> 318.
@@ -452,12 +458,23 @@ struct ScoreShape {
     int code, tile_w;
 };
 
-// c, and in *side_px D + 2w
-double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L, double *side_px = nullptr) {
+// Camera depth of the middle of a mesh's box under pose [16].
+float box_depth(const MeshRec &m, const float *pose) {
+    return 0.5f * (pose[8] * (m.lo[0] + m.hi[0]) + pose[9] * (m.lo[1] + m.hi[1]) + pose[10] * (m.lo[2] + m.hi[2])) + pose[11];
+}
+
+// Of the grid centre of a batched enumeration's item, or of its object's scene pose.
+float item_depth(const b3d_c2f_item &it) {
+    return it.centre_dev ? it.scene->obj_z[it.obj_slot] : box_depth(it.scene->meshes[it.scene->obj_mesh[it.obj_slot]], it.centre_pose);
+}
+
+// c for the object at camera depth z_obj, and in *side_px D + 2w; NaN where z_obj tells nothing
+double score_cost(const b3d_ctx *ctx, int32_t slot, const Lik &L, float z_obj, double *side_px = nullptr) {
     const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
     double d2 = 0;
     for (int k = 0; k < 3; ++k) d2 += (double)(m.hi[k] - m.lo[k]) * (m.hi[k] - m.lo[k]);
-    const double z = std::max((double)ctx->obj_z[slot], 0.5 * std::sqrt(d2) + ctx->cam.near_z);
+    const double z = z_obj;
+    if (!(z > 0.5 * std::sqrt(d2) + ctx->cam.near_z)) return NAN;
     const double f = std::max(ctx->cam.fx, ctx->cam.fy), side = 2.0 * L.w + 1.0;
     const double px2 = std::min(d2 * f * f / (z * z), (double)ctx->cam.W * ctx->cam.H);
     if (side_px) *side_px = std::sqrt(px2) + 2.0 * L.w;
@@ -468,27 +485,29 @@ int auto_tile_w(int cta_threads) { return cta_threads == 256 ? 128 : (cta_thread
 
 // large: the footprints do not fit the z-buffer of 128 threads
 ScoreShape shape_of_cost(double cost, bool large, int64_t n) {
-    const int64_t want = 152 * 600;  // threads that keep the device busy
+    const int64_t want = (int64_t)sm_count() * 600;  // threads that keep the device busy
     int nt = cost <= 1.3 ? 32 : (cost <= 2.6 ? 64 : (large ? 256 : 128));
     while (nt < 256 && n * nt < want) nt *= 2;
     const int code = nt == 128 ? 1 : (nt == 64 ? 2 : (nt == 32 ? 3 : 0));
     return ScoreShape{code << 8, auto_tile_w(nt)};
 }
 
-ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, int64_t n) {
+ScoreShape pick_shape(const b3d_ctx *ctx, int32_t slot, const Lik &L, float z_obj, int64_t n) {
+    const ScoreShape general{ctx->score_code(), ctx->tile_w};
     const MeshRec &m = ctx->meshes[ctx->obj_mesh[slot]];
     // half windows without a compiled-in scorer (an FP32 sum in the shape's order) and triangle
     // meshes keep the general shape
-    if (ctx->shape_set || m.n_quads <= 0 || L.w < 1 || L.w > 2) return ScoreShape{ctx->score_code(), ctx->tile_w};
+    if (ctx->shape_set || m.n_quads <= 0 || L.w < 1 || L.w > 2) return general;
     double side = 0;
-    const double cost = score_cost(ctx, slot, L, &side);
-    return shape_of_cost(cost, side > 63.0, n);
+    const double cost = score_cost(ctx, slot, L, z_obj, &side);
+    return std::isnan(cost) ? general : shape_of_cost(cost, side > 63.0, n);
 }
 
 // The shape of one batched launch: of the cost of a hypothesis, weighted by the time its scene
-// takes. slot(i), lik(i) and n(i): scene, slot, likelihood and hypotheses of item i.
-template <class Scene, class Slot, class Hyps>
-ScoreShape pick_shape_multi(const b3d_ctx *owner, int n_items, Scene scene, Slot slot, Hyps hyps, const std::vector<Lik> &Ls) {
+// takes. scene(i), slot(i), depth(i) and hyps(i): scene, slot, depth and hypotheses of item i.
+template <class Scene, class Slot, class Depth, class Hyps>
+ScoreShape pick_shape_multi(const b3d_ctx *owner, int n_items, Scene scene, Slot slot, Depth depth, Hyps hyps,
+                            const std::vector<Lik> &Ls) {
     const ScoreShape set{owner->score_code(), owner->tile_w};
     if (owner->shape_set) return set;
     double t = 0, tc = 0;
@@ -496,7 +515,8 @@ ScoreShape pick_shape_multi(const b3d_ctx *owner, int n_items, Scene scene, Slot
     for (int i = 0; i < n_items; ++i) {
         const b3d_ctx *sc = scene(i);
         if (sc->meshes[sc->obj_mesh[slot(i)]].n_quads <= 0 || Ls[i].w < 1 || Ls[i].w > 2) return set;
-        const double c = score_cost(sc, slot(i), Ls[i]);
+        const double c = score_cost(sc, slot(i), Ls[i], depth(i));
+        if (std::isnan(c)) return set;
         t += c * (double)hyps(i);
         tc += c * c * (double)hyps(i);
         total += hyps(i);
@@ -1223,7 +1243,7 @@ b3d_status b3d_set_scene(b3d_ctx *ctx, const b3d_intrinsics *intr, int32_t n_obj
     ctx->cam = c;
     ctx->obj_mesh.assign(mesh_ids, mesh_ids + n_obj);
     ctx->obj_z.resize(n_obj);
-    for (int32_t k = 0; k < n_obj; ++k) ctx->obj_z[k] = poses[16 * k + 11];
+    for (int32_t k = 0; k < n_obj; ++k) ctx->obj_z[k] = box_depth(ctx->meshes[mesh_ids[k]], poses + 16 * k);
     ctx->tri_base.assign(n_obj, 0);
     for (int32_t k = 1; k < n_obj; ++k) ctx->tri_base[k] = ctx->tri_base[k - 1] + ctx->meshes[mesh_ids[k - 1]].n_faces;
     {
@@ -1263,6 +1283,7 @@ b3d_status b3d_set_object_pose_dev(b3d_ctx *ctx, int32_t obj, const float *pose_
     cudaError_t e = cudaMemcpyAsync(ctx->d_poses + 16 * obj, pose_dev, 16 * sizeof(float), cudaMemcpyDeviceToDevice,
                                     (cudaStream_t)stream);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "set_object_pose_dev");
+    ctx->obj_z[obj] = NAN;
     bg_invalidate(ctx, obj);
     return B3D_OK;
 }
@@ -1310,7 +1331,7 @@ b3d_status b3d_score_batch(b3d_ctx *ctx, int32_t obj_slot, int64_t n_hyp, const 
         Timed tm(ctx, B3D_K_SCORE, s);
         SceneView sv = scene_view(ctx, obj_slot);
         sv.work = take_work(ctx);
-        const ScoreShape shape = pick_shape(ctx, obj_slot, L, n_hyp);
+        const ScoreShape shape = pick_shape(ctx, obj_slot, L, ctx->obj_z[obj_slot], n_hyp);
         sv.tile_w = shape.tile_w;
         launch_score_list(sv, L, PoseList{poses_dev}, n_hyp, loglik_dev, shape.code, s);
     }
@@ -1546,7 +1567,7 @@ b3d_status b3d_enumerate_c2f(b3d_ctx *ctx, int32_t obj_slot, const float *centre
         P.step = sch->stage[t].step;
         {
             Timed tm(ctx, B3D_K_SCORE, s);
-            const ScoreShape shape = pick_shape(ctx, obj_slot, L, n_t[t]);
+            const ScoreShape shape = pick_shape(ctx, obj_slot, L, box_depth(ctx->meshes[ctx->obj_mesh[obj_slot]], centre_pose), n_t[t]);
             sv.tile_w = shape.tile_w;
             launch_score_grid(sv, L, P, n_t[t], ctx->d_ll, shape.code, s);
         }
@@ -1611,7 +1632,7 @@ b3d_status b3d_score_multi(b3d_ctx *owner, int32_t n_items, const b3d_score_item
     });
     const ScoreShape shape = pick_shape_multi(
         owner, n_items, [&](int i) { return items[i].scene; }, [&](int i) { return items[i].obj_slot; },
-        [&](int i) { return items[i].n_hyp; }, Ls);
+        [&](int i) { return items[i].scene->obj_z[items[i].obj_slot]; }, [&](int i) { return items[i].n_hyp; }, Ls);
     const size_t off_items = 0, off_begin = align16(sizeof(BatchItem) * n_items);
     const size_t bytes = off_begin + align16(sizeof(int64_t) * (n_items + 1));
     unsigned char *h = nullptr;
@@ -1743,6 +1764,7 @@ b3d_status b3d_enumerate_multi(b3d_ctx *owner, int32_t n_items, const b3d_c2f_it
         int *bb = reinterpret_cast<int *>(h + o_bb) + (size_t)t * (n_items + 1);
         const ScoreShape shape = pick_shape_multi(
             owner, n_items, [&](int i) { return items[i].scene; }, [&](int i) { return items[i].obj_slot; },
+            [&](int i) { return item_depth(items[i]); },
             [&](int i) { return nh[(size_t)i * T + t]; }, Ls);
         codes[t] = shape.code;
         int64_t acc = 0;

@@ -266,6 +266,8 @@ int launch_bg_noise_tables(const SceneView &sv, const NoiseLik &N, float *nell, 
 void launch_score_noise(const SceneView &sv, const NoiseLik &N, const float *poses, int64_t n_hyp, const float *nell,
                         const double *nsums, float *out_ll, float *out_marg, cudaStream_t s);
 
+int sm_count();  // of the device
+
 // Context hooks used by the tracking server (defined with the context in b3d_api.cu).
 uint64_t ctx_used_bytes(b3d_ctx *ctx);
 void ctx_fix_shape(b3d_ctx *ctx);  // the score kernel keeps its default launch shape

@@ -470,7 +470,7 @@ int kernel_ctas_per_sm_impl(const void *kernel, int threads, int smem) {
     return per_sm;
 }
 
-static int sm_count() {
+int sm_count() {
     static int n = 0;
     if (!n) {
         int dev = 0;
