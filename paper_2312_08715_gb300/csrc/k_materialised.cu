@@ -488,7 +488,8 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
         if (x1 >= 0) {
             const int sx0 = max(x0 - w, 0), sx1 = min(x1 + w, c.W - 1);
             const int sy0 = max(y0 - w, 0), sy1 = min(y1 + w, c.H - 1);
-            const int tw = min(min(sx1 - sx0 + 1, min(S.tile_w, NT)), REG / (1 + 2 * w) - 2 * w);
+            // the column scorers give each column of a tile a thread
+            const int tw = min(min(sx1 - sx0 + 1, WT > 0 ? min(S.tile_w, NT) : S.tile_w), REG / (1 + 2 * w) - 2 * w);
             const int th = max(1, REG / (tw + 2 * w) - 2 * w);
             // the depths of the tile at (tx0, ty0) + w into dst
             auto stage = [&](int tx0, int ty0, float *dst) {

@@ -363,7 +363,8 @@ struct ScoreShared {
 // TAGS: the z-buffer holds 64-bit keys (depth bits, tag) in zb's memory (kRegionPx of them),
 // the tag being the rectangle's face class or the triangle's global id; the composite writes
 // the depths to zdt and the winning tags to tagt (-1 where the fixed objects are nearer).
-template <bool STATS, int NT, bool TAGS = false, class Visit>
+// COLS > 0: no tile is wider than COLS pixels (of a visitor that gives each column a thread).
+template <bool STATS, int NT, bool TAGS = false, int COLS = 0, class Visit>
 __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss_mode, ScoreShared<NT> &sh,
                                              float4 *s_stage, unsigned *zb, float4 *lat, unsigned long long *cnt,
                                              Visit &&visit, float *zdt = nullptr, int *tagt = nullptr) {
@@ -474,9 +475,8 @@ __device__ __forceinline__ bool render_tiles(const SceneView &S, int w, int miss
     const int sx0 = max(bx0 - w, 0), sx1 = min(bx1 + w, c.W - 1);
     const int sy0 = max(by0 - w, 0), sy1 = min(by1 + w, c.H - 1);
     const int sw = sx1 - sx0 + 1;
-    // the tile plus its halo must fit the region even one row high: (tw + 2w)(1 + 2w) <= REG;
-    // the column scorers give each column of a tile a thread
-    const int tw = min(min(sw, TAGS ? S.tile_w : min(S.tile_w, NT)), REG / (1 + 2 * w) - 2 * w);
+    // the tile plus its halo must fit the region even one row high: (tw + 2w)(1 + 2w) <= REG
+    const int tw = min(min(sw, COLS > 0 ? min(S.tile_w, COLS) : S.tile_w), REG / (1 + 2 * w) - 2 * w);
     const int th = max(1, div_small(REG, tw + 2 * w) - 2 * w);
     for (int ty0 = sy0; ty0 <= sy1; ty0 += th) {
         for (int tx0 = sx0; tx0 <= sx1; tx0 += tw) {
@@ -784,7 +784,7 @@ __device__ __forceinline__ double score_body(const SceneView &S, const Lik &L, c
         sh.fix[0] = sh.fix[1] = 0;
         sh.wild = 0.f;
     }
-    const bool drawn = render_tiles<STATS, NT>(
+    const bool drawn = render_tiles<STATS, NT, false, (WT > 0 ? NT : 0)>(
         S, w, L.miss_mode, sh, s_stage, zb, lat, cnt,
         [&](const float *zd, int zx0, int zy0, int zw, int qx0, int qx1, int qy0, int qy1, int, int, int, int) {
             const int tww = qx1 - qx0 + 1, thh = qy1 - qy0 + 1;
