@@ -20,6 +20,11 @@ __device__ __forceinline__ float warp_sum(float v) {
     return v;
 }
 
+// A term's or derivative's difference from the background's, rounded as it stands: the compiler may
+// not fold the term's last product into it, since equal terms have to give 0 (in the gradient
+// kernel they left a part in 10^8 of each term where an object is hidden).
+__device__ __forceinline__ float minus_bg(float v, float bg) { return __fsub_rn(v, bg); }
+
 // Block-wide sum over kThreads threads; result valid in thread 0. Uses red[kThreads/32].
 __device__ __forceinline__ float block_sum(float v, float *red) {
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;

@@ -146,9 +146,10 @@ __global__ void __launch_bounds__(NT, kGradMinBlocks)
                                                 l, gs, gp, bp);
                             }
                             if (x >= tx0 && x <= tx1 && y >= ty0 && y <= ty1) {
-                                acc_l += l - S.ell_bg[gi];
-                                acc_s += gs - S.gs_bg[gi];
-                                acc_p += gp - S.gp_bg[gi];
+                                // rounded as they stand (see minus_bg): 0 where nothing changed
+                                acc_l += minus_bg(l, S.ell_bg[gi]);
+                                acc_s += minus_bg(gs, S.gs_bg[gi]);
+                                acc_p += minus_bg(gp, S.gp_bg[gi]);
                             }
                         }
                         ipq[k] = make_float2(bp * wscale, q.z);

@@ -569,9 +569,9 @@ __global__ void __launch_bounds__(NT, MINB) k_score_fused(SceneView S, Lik L, co
                             const int64_t gi = (int64_t)gy * c.W + gx;
                             const float4 q = S.obs[gi];
                             if (q.w != 0.f)
-                                acc += pixel_ell(L, s_lut, c, q, gx, gy,
-                                                 [&](int xj, int yj) { return zd[(yj - zy0) * zw + (xj - zx0)]; }) -
-                                       S.ell_bg[gi];
+                                acc += minus_bg(pixel_ell(L, s_lut, c, q, gx, gy,
+                                                          [&](int xj, int yj) { return zd[(yj - zy0) * zw + (xj - zx0)]; }),
+                                                S.ell_bg[gi]);
                             x += dr;
                             y += dq;
                             if (x >= tww) { x -= tww; ++y; }

@@ -284,9 +284,7 @@ __device__ __forceinline__ void score_column_kind(const SceneView &S, const Lik 
         // a pixel without a point is skipped only now: a branch around the window loop costs
         // more than the loop (the lanes' pixels diverge)
         if (qe.x == 0.f) continue;
-        // rounded as it stands: the compiler may not fold the logarithm's last product into the
-        // difference, which is 0 for a term equal to the background's
-        sum.add(__fsub_rn(l, qe.y), KIND == 1);
+        sum.add(minus_bg(l, qe.y), KIND == 1);
         if (n_px) {
             ++*n_px;
             *n_pairs += (unsigned long long)((min(y + W, c.H - 1) - max(y - W, 0) + 1) *
@@ -826,7 +824,7 @@ __device__ __forceinline__ double score_body(const SceneView &S, const Lik &L, c
                         }
                         const float l = pixel_ell(L, s_lut, c, q, gx, gy,
                                                   [&](int xj, int yj) { return zd[(yj - zy0) * zw + (xj - zx0)]; });
-                        acc += l - S.ell_bg[gi];
+                        acc += minus_bg(l, S.ell_bg[gi]);
                     }
                     x += dr;
                     y += dq;

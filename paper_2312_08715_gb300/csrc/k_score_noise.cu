@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(NT, MINB)
                                     [&](int xj, int yj) { return zd[(yj - zy0) * zw + (xj - zx0)]; }, l, &counts);
 #pragma unroll
                         for (int g = 0; g < kMaxNoise; ++g)
-                            if ((g >> 2) < N.nr && (g & 3) < N.np) acc[g] += l[g] - nell[(int64_t)g * npx + gi];
+                            if ((g >> 2) < N.nr && (g & 3) < N.np) acc[g] += minus_bg(l[g], nell[(int64_t)g * npx + gi]);
                     }
                     x += dr;
                     y += dq;
