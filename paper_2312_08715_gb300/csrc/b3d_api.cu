@@ -36,6 +36,7 @@ struct MeshRec {
     int *class_off = nullptr, *tri_off = nullptr;
     float *coords = nullptr;
     int n_quads = 0, nc[3] = {0, 0, 0}, np1 = 0;
+    float gap = 0.f;
 };
 
 struct LikKey {
@@ -322,6 +323,7 @@ MeshView view_of(const MeshRec &m) {
     v.tri_off = m.tri_off;
     v.coords = m.coords;
     v.np1 = m.np1;
+    v.gap = m.gap;
     return v;
 }
 
@@ -1154,6 +1156,11 @@ b3d_status b3d_load_mesh(b3d_ctx *ctx, const float *verts, int64_t n_v, const in
     rec.n_quads = (int)h_quads.size();
     for (int k = 0; k < 3; ++k) rec.nc[k] = nc[k];
     rec.np1 = np1;
+    if (rec.n_quads > 0) {
+        rec.gap = INFINITY;
+        for (int a = 0, k = 0; a < 3; k += nc[a++])
+            for (int i = 1; i < nc[a]; ++i) rec.gap = std::min(rec.gap, h_coords[k + i] - h_coords[k + i - 1]);
+    }
 
     DeviceGuard g(ctx->device);
     b3d_status st = B3D_OK;

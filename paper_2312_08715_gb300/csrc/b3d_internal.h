@@ -63,6 +63,7 @@ struct MeshView {
     int nc[3];                  // planes per axis
     int np1;                    // stride of class_off and tri_off (max planes + 1)
     const int *tri_off;         // [6 * (np1)]: first surface triangle of class c with plane >= p, or NULL
+    float gap;                  // smallest distance of neighbouring lattice planes
 };
 
 // Windowed likelihood constants (Eq. 1 with the window of Sec. III-B).

@@ -117,7 +117,7 @@ __device__ __forceinline__ void cam_raster(const CamObject *obj, const int *orde
 // Depth and ids (64-bit keys), or depths of images whose z-buffer does not fit in shared
 // memory: screen tiles of kRegionPx pixels. Scenes of any number of objects, kMaxCamObjects
 // at a time.
-__global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshView *meshes, const int *tri_base,
+__global__ void __launch_bounds__(kThreads, 3) k_render_camera(Cam c, const MeshView *meshes, const int *tri_base,
                                                             const float *world, int n_obj, PoseList P, int64_t n_hyp,
                                                             float *out_depth, int *out_tid) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -169,7 +169,7 @@ __global__ void __launch_bounds__(kThreads) k_render_camera(Cam c, const MeshVie
 // one pass over each object's triangles per hypothesis (the tiled kernel above sets every
 // triangle up once per screen tile).
 template <int NT>
-__global__ void __launch_bounds__(NT) k_render_camera_depth(Cam c, const MeshView *meshes, const float *world,
+__global__ void __launch_bounds__(NT, NT == 256 ? 3 : 1) k_render_camera_depth(Cam c, const MeshView *meshes, const float *world,
                                                             int n_obj, PoseList P, int64_t n_hyp, float *out_depth) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned *zb = reinterpret_cast<unsigned *>(smem_raw);  // [W H] depth bits

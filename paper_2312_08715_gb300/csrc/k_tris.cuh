@@ -85,11 +85,29 @@ struct TriRanges {
 // Screen box, flags (bit 0: on screen, bit 2: whole object beyond the near plane) and triangle
 // ranges of one object under pose P (shared memory), by one warp. The ranges of a mesh whose
 // surface triangles are stored by class hold every triangle of a class whose plane has the
-// camera on its outer side, with a margin: planes within kFaceMargin of the camera's distance
-// are kept, and the screen-area test of tri_setup decides, as it does without ranges (a plane
-// farther inside than the margin has a screen area whose sign is far above its rounding).
-// A pose far from a rigid one takes every triangle.
+// camera on its outer side, and those of planes at most a margin farther in, whose triangles the
+// screen-area test of tri_setup decides on as it does without ranges. The margin is where the sign
+// of that area cannot be its rounding's (see face_margin); 1 to 3 mm for 5 mm cells under a
+// of 160x120. A pose that is not rigid to some percent takes every triangle.
+//
+// A triangle of legs e_b, e_c on a plane that the camera is d farther in than has twice the screen
+// area f^2 e_b e_c d / (z_a z_b z_c). What is computed differs by the rounding of its vertices,
+// each coordinate by E <= 2^-24 (3 f S / z + 3 V (1 + S / z)) with S the largest sum in the
+// transform and V the largest screen coordinate (beyond the image too, with the principal point's),
+// so by 2 sqrt(2) E (f + V) (e_b + e_c) / z + 8 E^2, and by 3 2^-24 of the squared leg (f + V) e / z
+// in the products. With the smallest gap e of the lattice, K = 1 + V / f and r = E z / (f e) the
+// sign is certain beyond d = z (5.7 K r + 8 r^2 + 3 2^-24 K^2), which grows with z: the farthest
+// corner's is taken, and a third more for poses that are rigid to some percent only. kFaceMargin
+// covers the rounding of the camera's position.
 constexpr float kFaceMargin = 1e-4f;
+__device__ __forceinline__ float face_margin(const MeshView &m, const Cam &c, float dist, float z, float screen) {
+    const float rx = fmaxf(fabsf(m.lo[0]), fabsf(m.hi[0])), ry = fmaxf(fabsf(m.lo[1]), fabsf(m.hi[1]));
+    const float rad = sqrtf(rx * rx + ry * ry + fmaxf(m.lo[2] * m.lo[2], m.hi[2] * m.hi[2]));  // of the box's corners
+    const float S = dist + 2.f * rad, zf = 1.05f * (z + rad), f = fminf(c.fx, c.fy), fm = fmaxf(c.fx, c.fy);
+    const float V = screen + fmaxf(fabsf(c.cx), fabsf(c.cy)), K = (fm + V) / f;
+    const float r = 0x1p-24f * 3.f * (fm * S + V * (zf + S)) / (f * m.gap);  // E z / (f e)
+    return kFaceMargin * (1.f + dist) + 1.34f * zf * (r * fmaf(8.f, r, 5.7f * K) + 3.f * 0x1p-24f * K * K);
+}
 __device__ __forceinline__ void tri_view_warp(const MeshView &m, const float *P, const Cam &c, int lane, int *bb,
                                               int *flags, TriRanges *rg) {
     float umin = INFINITY, umax = -INFINITY, vmin = INFINITY, vmax = -INFINITY;
@@ -125,12 +143,18 @@ __device__ __forceinline__ void tri_view_warp(const MeshView &m, const float *P,
                     cz = P[i] * P[3 + j] - P[3 + i] * P[j];
         const float det = fmaf(P[a], cx, fmaf(P[3 + a], cy, P[6 + a] * cz));
         const float t2 = fmaf(P[9], P[9], fmaf(P[10], P[10], P[11] * P[11]));
-        const float oa = -fmaf(cx, P[9], fmaf(cy, P[10], cz * P[11])) / det, marg = kFaceMargin * (1.f + sqrtf(t2));
+        const float oa = -fmaf(cx, P[9], fmaf(cy, P[10], cz * P[11])) / det;
+        const float marg = face_margin(m, c, sqrtf(t2), P[11],
+                                       fmaxf(fmaxf(fabsf(umin), fabsf(umax)), fmaxf(fabsf(vmin), fabsf(vmax))));
+        // squared lengths of the rotation's columns
+        float col = 0.f;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) col = fmaxf(col, fmaf(P[k], P[k], fmaf(P[3 + k], P[3 + k], P[6 + k] * P[6 + k])));
         const int *off = m.tri_off + lane * m.np1;
         const int n = m.nc[a];
         const float *cd = m.coords + (a == 0 ? 0 : (a == 1 ? m.nc[0] : m.nc[0] + m.nc[1]));
         int lo = 0, hi = n;
-        if (!(det > 0.5f && det < 2.f)) {
+        if (!(det > 0.95f && det < 1.05f && col < 1.05f)) {
             b = off[0];
             cnt = off[n] - b;
         } else if (lane & 1) {  // outward +axis: planes below the camera
