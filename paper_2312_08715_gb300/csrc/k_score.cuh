@@ -52,7 +52,8 @@ inline int score_sm_count() {
 //     triangle id rides along), score the tile's observed pixels against their background terms.
 //  4. block reduction to one log-likelihood (FixedSum: the same bits under every launch shape).
 // STATS: count the work done (hypotheses, projected vertices/corners, primitives, pixel
-// tests, fragments, composited pixels, scored pixels, window pairs) into S.stats.
+// tests, fragments, composited pixels (a tile's and its halo's, which start from the background),
+// scored pixels, window pairs) into S.stats.
 // WT: the half window compiled in (1 or 2: sliding-window scoring), 0: runtime L.w.
 
 // Screen corner of a camera-frame point; approximate reciprocal (the same bits for the same
