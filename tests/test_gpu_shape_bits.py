@@ -60,14 +60,15 @@ def test_scores_are_the_same_bits(orc, width, vox, lik):
         c.close()
 
 
-def test_untuned_enumerations_equal_batched_ones(orc):
-    """Particles, weights and densities of two scenes of very different size, whose single calls
-    and whose batch take different launch shapes."""
+@pytest.mark.parametrize("scenes,n_rot", [([(64, 500), (320, 9000), (97, 1500)], 9), ([(64, 500), (72, 700)], 40)])
+def test_untuned_enumerations_equal_batched_ones(orc, scenes, n_rot):
+    """Particles, weights and densities of scenes whose single calls and whose batch take different
+    launch shapes: uneven ones (256 threads for the batch), and small ones of many hypotheses (32)."""
     from paper_2312_08715_gb300 import b3d
-    stages = [synth.StageSpec(7, 0.01, 1, 9, math.radians(6)), synth.StageSpec(9, 0.003, 1, 3, math.radians(2))]
+    stages = [synth.StageSpec(7, 0.01, 1, n_rot, math.radians(6)), synth.StageSpec(9, 0.003, 1, 3, math.radians(2))]
     lik, M = dict(kind=0, radius=0.004, p_outlier=0.02, half_window=1), 24
     owner, ctxs, items, singles, outs = b3d.Context(0), [], [], [], []
-    for k, (width, vox) in enumerate([(64, 500), (320, 9000), (97, 1500)]):
+    for k, (width, vox) in enumerate(scenes):
         wl, obs = _scene(orc, width, vox, seed=20 + k)
         ctx = gpu_context(wl.scene, obs)
         centre = wl.hidden.astype(np.float32)
