@@ -460,14 +460,9 @@ struct ScoreShape {
     int code, tile_w;
 };
 
-// Camera depth of the middle of a mesh's box under pose [16].
-float box_depth(const MeshRec &m, const float *pose) {
-    return 0.5f * (pose[8] * (m.lo[0] + m.hi[0]) + pose[9] * (m.lo[1] + m.hi[1]) + pose[10] * (m.lo[2] + m.hi[2])) + pose[11];
-}
-
-// Of the grid centre of a batched enumeration's item, or of its object's scene pose.
+// Camera depth of the grid centre of a batched enumeration's item, or of its object's scene pose.
 float item_depth(const b3d_c2f_item &it) {
-    return it.centre_dev ? it.scene->obj_z[it.obj_slot] : box_depth(it.scene->meshes[it.scene->obj_mesh[it.obj_slot]], it.centre_pose);
+    return it.centre_dev ? it.scene->obj_z[it.obj_slot] : it.centre_pose[11];
 }
 
 // c for the object at camera depth z_obj, and in *side_px D + 2w; NaN where z_obj tells nothing
@@ -1250,7 +1245,7 @@ b3d_status b3d_set_scene(b3d_ctx *ctx, const b3d_intrinsics *intr, int32_t n_obj
     ctx->cam = c;
     ctx->obj_mesh.assign(mesh_ids, mesh_ids + n_obj);
     ctx->obj_z.resize(n_obj);
-    for (int32_t k = 0; k < n_obj; ++k) ctx->obj_z[k] = box_depth(ctx->meshes[mesh_ids[k]], poses + 16 * k);
+    for (int32_t k = 0; k < n_obj; ++k) ctx->obj_z[k] = poses[16 * k + 11];
     ctx->tri_base.assign(n_obj, 0);
     for (int32_t k = 1; k < n_obj; ++k) ctx->tri_base[k] = ctx->tri_base[k - 1] + ctx->meshes[mesh_ids[k - 1]].n_faces;
     {
@@ -1574,7 +1569,7 @@ b3d_status b3d_enumerate_c2f(b3d_ctx *ctx, int32_t obj_slot, const float *centre
         P.step = sch->stage[t].step;
         {
             Timed tm(ctx, B3D_K_SCORE, s);
-            const ScoreShape shape = pick_shape(ctx, obj_slot, L, box_depth(ctx->meshes[ctx->obj_mesh[obj_slot]], centre_pose), n_t[t]);
+            const ScoreShape shape = pick_shape(ctx, obj_slot, L, centre_pose[11], n_t[t]);
             sv.tile_w = shape.tile_w;
             launch_score_grid(sv, L, P, n_t[t], ctx->d_ll, shape.code, s);
         }
