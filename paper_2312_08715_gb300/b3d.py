@@ -400,6 +400,8 @@ def b3d_get_tuning(ctx) -> dict:
 
 
 def b3d_set_tuning(ctx, tile_w=64, cta_threads=256, ctas_per_sm=0, high_occupancy=0, batch_chunk=4):
+    """Sets every field (those left out to the general default) and with them the launch shape,
+    which until then follows the size of the work."""
     return _check(ctx, load().b3d_set_tuning(ctx, C.byref(b3d_tuning(tile_w, cta_threads, ctas_per_sm,
                                                                        high_occupancy, batch_chunk))))
 

@@ -431,31 +431,28 @@ SceneView scene_view(b3d_ctx *ctx, int32_t slot) {
 }
 
 // Launch shape of a score launch (the code of launch_score and the tile width) when none was
-// set or tuned: single calls, each stage of an enumeration and batched launches, with half windows
-// whose scores do not depend on the shape (FixedSum in k_score.cuh). The CTA size follows the
-// work of a hypothesis, estimated in microseconds of an SM from the slot object's rectangles q and
-// its size D in pixels at the depth of the grid's centre where the host knows it, else of the
+// set or tuned: single calls, each stage of an enumeration and batched launches, with half
+// windows whose scores do not depend on the shape (FixedSum in k_score.cuh). The CTA size follows
+// the work of a hypothesis, estimated in microseconds of an SM from the slot object's rectangles q
+// and its size D in pixels at the depth of the grid's centre where the host knows it, else of the
 // scene's pose:
 //   c = 0.35 + 0.00113 q + D^2 (0.0003 + e (2w+1)^2), e = 0.00006 (ball) or 0.0001 (Gaussian),
 // a fit to a sweep of 33 shapes over 64x48 to 320x240 images, objects of 600 to 12,000 cells
-// and both likelihoods. Up to 1.3 us a hypothesis 32 threads are the fastest (30,000
-// hypotheses of 873 cells at 160x120: 175 us; 64: 205, 128: 236, 256: 398), up to 2.6 64
-// (5,109 cells, 160x120: 453; 128: 463, 256: 696), above 128, or 256 with tiles of 128 pixels
-// where the footprint does not fit the 3,072-pixel z-buffer of 128 threads and would be drawn
-// tile by tile. For one object that line lies at D + 2w = 63, whatever the likelihood (112
-// points of 64x48 to 320x240 images, objects of 800 to 15,000 cells; 3,000 hypotheses, us at
-// 128 and 256 threads: D = 59.5, w = 1 103 and 107; 62.8 119 and 108; 72 165 and 134; 58.6,
-// w = 2 127 and 145; 59.5 147 and 142; a line by c had cost 5x5 windows up to 18%); a batch of
-// scenes, whose sizes differ, takes 256 above c = 5.8. A call of few hypotheses takes
-// larger CTAs, so that each SM still has some 600 threads: 1,000 hypotheses of the first
-// object take 15 us with 128 threads, 24 with 256; 300 take 12 with 256, 13 with 64. Where the
+// and both likelihoods. Times of the kernels as they are, in us at 32 / 64 / 128 / 256 threads:
+// up to c = 1.3 32 threads (four 64x48 scenes of 24,064 hypotheses 1,399 / - / - / 2,041), up to
+// 2.6 64 (30,000 of 1,033 cells at 160x120: 307 / 298 / 312 / 449), above 128 (5,745 cells:
+// 614 / 496 / 486 / 693), or 256 with tiles of 128 pixels where the footprint does not fit the
+// 3,072-pixel z-buffer of 128 threads and would be drawn tile by tile. For one object that line
+// lies at D + 2w = 63 (3,000 hypotheses of 5,155 cells at 128 and 256 threads: w = 1, D = 57.2 78
+// and 95; 60.2 89 and 97; 62.2 98 and 99; 68.2 117 and 108; w = 2, D = 57.2 122 and 126; 59.2 128
+// and 130; 61.2 138 and 134; 64.2 155 and 138); a batch of scenes, whose sizes differ, takes 256
+// above c = 5.8. A call of few hypotheses takes larger CTAs, so that each SM still has some 600
+// threads: 1,000 of the 1,033-cell object take 34 / 22 / 19 / 28, 300 33 / 19 / 17 / 14. Where the
 // depth is not known (an object whose pose came from the device, or whose scene pose does not lie
 // before the camera: a placeholder) the general shape stays: a depth 16 times too large made a
 // search of 3,750 hypotheses of 600 cells 404 us long, the general shape takes 319 and the right
-// depth's 291.
-// Calls that kept 256 threads and 64-pixel tiles before: 1,000 hypotheses at 64x48 36 -> 26 us,
-// 16,001 smooth 5x5 ones at 150x113 470 -> 367, 31,250 at 320x240 1,569 -> 1,324, eight scenes
-// batched 721 -> 595, a tracking step at 320x240 370 -> 318.
+// depth's 291. Against the general shape: 1,000 hypotheses at 64x48 33 -> 27, 16,001 smooth 5x5
+// ones at 150x113 463 -> 367, eight scenes batched 557 -> 447, 31,250 at 320x240 1,187 either way.
 struct ScoreShape {
     int code, tile_w;
 };

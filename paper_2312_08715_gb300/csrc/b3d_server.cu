@@ -560,7 +560,7 @@ b3d_status b3d_server_create(b3d_server **out, int32_t device, uint64_t hbm_budg
         b3d_destroy(S->owner);
         return srv_fail(s2, m);
     };
-    ctx_fix_shape(S->owner);  // whatever frames share a batch
+    ctx_fix_shape(S->owner);  // for half windows whose sums follow it: whatever frames share a batch
     if (cfg->tuning.tile_w != 0 && (st = b3d_set_tuning(S->owner, &cfg->tuning)) != B3D_OK)
         return bail(st, std::string("tuning: ") + b3d_last_error(S->owner));
     // the batch scratch for max_batch_items items is reserved once, up front

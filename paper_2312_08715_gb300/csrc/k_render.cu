@@ -43,7 +43,8 @@ struct CamObject {
 // Objects of kCamLarge pixels of screen box a triangle and more go out 8 triangles to a batch
 // in CTAs of more than 8 warps: a warp tests such triangles one after another, and 32 of an
 // 800-triangle table were a warp's whole share of a hypothesis, at whose end the others waited
-// (2,048 hypotheses at 200x200: 1,154 -> 882 us, barrier stalls 7.0 -> 1.7 cycles an issue).
+// (2,048 hypotheses at 200x200, rendered and scored: 1,614 -> 1,368 us; barrier stalls 7.0 -> 1.7
+// cycles an issue).
 // With 24 as the line, or with 8 warps a CTA, the set-up by 8 lanes costs more than it evens
 // out (1,500 hypotheses of 150x150 867 -> 872 us, of 100x100 353 -> 357).
 constexpr float kCamLarge = 40.f;

@@ -14,7 +14,7 @@
 // two boxes, 800-triangle table) 3.78 -> 1.16 ms, 794k -> 326k warp instructions a hypothesis;
 // object render with ids, 2,048 poses at 160x120, 0.306 -> 0.119 ms, 75k -> 34k instructions.
 // What is left is instruction issue (set-up and pixel tests): with large triangles in batches
-// of 8 the camera render takes 0.88 ms at 69% of the issue rate. Pixels two at a time in packed
+// of 8 the camera render takes 0.93 to 1.0 ms at 69% of the issue rate. Pixels two at a time in packed
 // arithmetic, by a lane for its own triangle or by the warp, were no faster.
 #pragma once
 
